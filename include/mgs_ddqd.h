@@ -77,23 +77,28 @@ size_t mgs_workspace_bytes(int limbs, int m, int n, int with_rhs);
  * counterpart in the paper; for tests and tuning).  `out` has room for 5 ints.
  *   out[0] Br  row blocks (CTAs per column group), out[1] Bc  column groups,
  *   out[2] h   rows per row block, out[3] kernel:
- *     0  grid-barrier kernel: one grid-wide barrier per elimination step;
+ *     0  grid kernel: a plain cooperative grid.  Br = 1 (the default for limbs 2 and 4
+ *        where a CTA's columns fit in shared memory): whole columns per CTA, integer
+ *        arithmetic, no barrier between CTAs during the sweep.  Br > 1: row blocks, FP64
+ *        arithmetic, one grid-wide barrier per elimination step;
  *     1  cluster schedule on hardware thread-block clusters (the Br CTAs of a column
  *        group form one cluster and exchange Gram partials through distributed shared
  *        memory; Br <= 8);
  *     2  the same schedule on software groups (the Br CTAs meet at a counter in global
  *        memory and exchange partials through L2; every SM usable).
- *   The default is 1 for limbs 1 and 2 where the clusters fill at least 90 % of the SMs
- *   a plain grid would use (else 0), and 0 for limbs 4: measured on GB300, the cluster
- *   schedule hides the per-step latency that dominates the cheaper arithmetic, while quad
- *   double, and layouts where clusters leave SMs idle, are bound by FP64 throughput.
+ *   Where whole columns do not fit, and for limbs 1, the default is 1 for limbs 1 and 2
+ *   where the clusters fill at least 90 % of the SMs a plain grid would use, else 0.
  *   The environment variable MGS_KERNEL = grid | cluster | group, read at each call,
- *   forces a kernel (cluster falls back to grid where clusters cannot be formed);
- *   out[4] threads per CTA: 128, or 256 where a CTA owns 16 or more columns (two warps
- *          per SM sub-partition hide each other's FP64 latency in the long loops).
- *   MGS_ROWS = h overrides the rows per row block (default 64); MGS_CTA_THREADS = 128 |
+ *   forces a kernel with row blocks (cluster falls back to grid where clusters cannot be
+ *   formed);
+ *   out[4] threads per CTA of a kernel with row blocks: 128, or 256 where a CTA owns 16 or
+ *          more columns (two warps per SM sub-partition hide each other's FP64 latency in
+ *          the long loops).  The kernel with whole columns sizes its CTAs by the rows and
+ *          columns itself (up to 512 threads); this is then the value for its column count.
+ *   MGS_ROWS = h sets the rows per row block (64 without it); MGS_CTA_THREADS = 128 |
  *   256 the threads per CTA; MGS_CTAS_PER_SM = 1 | 2 how many CTAs of the solve share an
  *   SM (default 1: each has the SM's FP64 unit to itself; 2 doubles the column groups).
+ *   Any of them selects a kernel with row blocks.
  * Returns MGS_OK, MGS_EINVAL or MGS_ENOSPACE (no layout fits shared memory).
  */
 int mgs_plan_query(int limbs, int m, int n, int with_rhs, int* out);

@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "lib")
 LIBRARY = os.path.join(LIBDIR, "libmgs_ddqd.so")
 HOST_LIBRARY = os.path.join(LIBDIR, "libddqd_host.so")
-SOURCES = ["api.cu", "mgs_d.cu", "mgs_dd.cu", "mgs_qd.cu", "noalloc.cu", "batched.cu", "newton.cu", "probe.cu"]
+SOURCES = ["api.cu", "mgs_d.cu", "mgs_dd.cu", "mgs_qd.cu", "mgs_column.cu", "noalloc.cu", "batched.cu", "newton.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--fmad=false"]
 # extra nvcc flags for experiments; empty by default
@@ -77,7 +77,7 @@ def build_host(force: bool = False) -> str:
     """Host build of the device arithmetic (csrc/ddqd.cuh as plain C++) for the CPU tests."""
     os.makedirs(LIBDIR, exist_ok=True)
     src = os.path.join(CSRC, "ddqd_host.cpp")
-    deps = [src, os.path.join(CSRC, "ddqd.cuh")]
+    deps = [src, os.path.join(CSRC, "ddqd.cuh"), os.path.join(CSRC, "wide.cuh")]
     if not force and os.path.exists(HOST_LIBRARY) and all(
             os.path.getmtime(d) <= os.path.getmtime(HOST_LIBRARY) for d in deps):
         return HOST_LIBRARY

@@ -10,6 +10,7 @@
 
 #include "../../include/mgs_ddqd.h"
 #include "launch.cuh"
+#include "mgs_column.cuh"
 
 namespace mgs {
 int launch_cluster_d(const Params& pr, int grid, int cl, int T, size_t smem, cudaStream_t stream);
@@ -26,6 +27,8 @@ int launch_cluster(int L, const Params& pr, int grid, int cl, int T, size_t smem
 int cluster_capacity(int L, int cl, int T, size_t smem) {
   return L == 1 ? cluster_capacity_d(cl, T, smem) : L == 2 ? cluster_capacity_dd(cl, T, smem) : cluster_capacity_qd(cl, T, smem);
 }
+int column_capacity(int L, int threads, size_t smem);
+int launch_column(int L, const ColParams& pr, int threads, size_t smem, cudaStream_t stream);
 int blocks_per_sm_d(int kind, int T, size_t smem);
 int blocks_per_sm_dd(int kind, int T, size_t smem);
 int blocks_per_sm_qd(int kind, int T, size_t smem);
@@ -49,6 +52,9 @@ struct Plan {
   int T;     // threads per CTA (128 or 256)
   size_t smem;
   size_t off_sync, off_gsync, off_flags, off_P, off_V, off_Y, off_R, off_G, off_T, total, zero_bytes;
+  // the column kernel (col != 0): panel width, warps on columns, pivot stages, column k+1 first
+  int col, bw, warps, stages, first;
+  size_t off_C, off_Rd;
 };
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -156,12 +162,66 @@ bool compute_plan(int L, int m, int n, int aug, int want, int h0, int T0, int cp
   off = align256(off + sizeof(double) * (size_t)n * n * E);
   pl.off_G = off;  // G_kk, r_kk, 1/r_kk
   off = align256(off + sizeof(double) * 3 * (size_t)pl.nc * L);
+  pl.col = 0;
   pl.off_T = off;
 #if defined(MGS_TRACE) && MGS_TRACE
   off = align256(off + sizeof(unsigned long long) * 8 * (size_t)(pl.nc + 1) * pl.Br * pl.Bc);
 #endif
   pl.total = off;
   return true;
+}
+
+// The column kernel's layout (double-double and quad-double, default choices only): whole
+// columns per CTA.  Replaces the plan made before it when a CTA's columns and two pivot
+// stages fit in shared memory; the workspace stays at least what that plan asked for.
+void column_plan(Plan& pl) {
+  const int L = pl.L, m = pl.m, nc = pl.nc;
+  if (L == 1 || m > 2048) return;
+  const int sms = device_sms();
+  int bw = 1, warps = mgs::kColWarps, stages = 4, first = 1;
+  int Bc = nc < sms ? nc : sms;
+  const int halves = (m + 15) / 16;  // 16-row pieces of a column
+  if (Bc > (nc + bw - 1) / bw) Bc = (nc + bw - 1) / bw;
+  const int w = (nc + bw * Bc - 1) / (bw * Bc) * bw;
+  if (warps > halves * (w + 1)) warps = halves * (w + 1);  // a pass: w columns and the norm
+  size_t smem;
+  for (;; --stages) {
+    if (stages < 2) return;
+    smem = mgs::col_smem_bytes(L, m, w, stages);
+    const size_t bs = mgs::col_backsub_bytes(L, pl.n);
+    if (bs > smem) smem = bs;
+    if (smem <= kMaxSmem) break;
+  }
+  const size_t pad = cta_per_sm_smem(1);
+  if (pad > smem && pad <= kMaxSmem) smem = pad;
+  const int threads = 32 * (warps + 1);
+  if (mgs::column_capacity(L, threads, smem) * sms < Bc) return;
+  pl.col = 1;
+  pl.kind = 0;
+  pl.Br = 1;
+  pl.Bc = Bc;
+  pl.h = m;
+  pl.w = w;
+  pl.bw = bw;
+  pl.warps = warps;
+  pl.stages = stages;
+  pl.first = first;
+  pl.T = (nc + Bc - 1) / Bc >= 16 ? 256 : 128;
+  pl.smem = smem;
+  size_t off = 64;
+  pl.off_sync = 0;
+  pl.off_flags = off;
+  off = align256(off + sizeof(unsigned) * (size_t)nc);
+  pl.zero_bytes = off;
+  pl.off_Rd = off;
+  off = align256(off + sizeof(double) * (size_t)nc * L);
+  pl.off_C = off;
+  off = align256(off + sizeof(double) * (size_t)nc * (nc - 1) / 2 * 2 * L);
+#if defined(MGS_TRACE) && MGS_TRACE
+  pl.off_T = off;
+  off = align256(off + sizeof(unsigned long long) * 8 * (size_t)(nc + 1) * Bc);
+#endif
+  if (off > pl.total) pl.total = off;
 }
 
 // The plan for (device, sizes, kernel choice), computed once: it queries occupancy, which
@@ -199,6 +259,7 @@ bool make_plan(int L, int m, int n, int aug, Plan& pl) {
       }
   }
   if (!compute_plan(L, m, n, aug, want, h, T, cps, pl)) return false;
+  if (want < 0 && !henv && T == 0 && cps == 1) column_plan(pl);
   std::lock_guard<std::mutex> g(mu);
   if (cache.size() >= 256) cache.clear();
   cache.push_back(Entry{dev, L, m, n, aug, want, h, T, cps, pl});
@@ -227,6 +288,42 @@ int run(int L, double* A, int lda, double* b, double* x, double* R, int ldr, dou
   if (e != cudaSuccess) {
     g_last_cuda = (int)e;
     return MGS_ECUDA;
+  }
+  if (pl.col) {
+    mgs::ColParams cp{};
+    cp.A = A;
+    cp.lda = lda;
+    cp.b = aug ? b : nullptr;
+    cp.R = R;
+    cp.ldr = ldr;
+    cp.x = aug ? x : nullptr;
+    cp.z = aug ? z : nullptr;
+    cp.m = m;
+    cp.n = n;
+    cp.nc = pl.nc;
+    cp.aug = pl.aug;
+    cp.Bc = pl.Bc;
+    cp.bw = pl.bw;
+    cp.w = pl.w;
+    cp.warps = pl.warps;
+    cp.stages = pl.stages;
+    cp.first = pl.first;
+    cp.C = reinterpret_cast<mgs::u32*>(wb + pl.off_C);
+    cp.Rd = reinterpret_cast<mgs::u32*>(wb + pl.off_Rd);
+    cp.flags = reinterpret_cast<unsigned*>(wb + pl.off_flags);
+    cp.sync = reinterpret_cast<unsigned*>(wb + pl.off_sync);
+    cp.status = dev_status;
+    cp.timeout_ns = kTimeoutNs;
+    cp.skip = skip;
+#if defined(MGS_TRACE) && MGS_TRACE
+    cp.trace = reinterpret_cast<unsigned long long*>(wb + pl.off_T);
+#endif
+    const int rc = mgs::launch_column(L, cp, 32 * (pl.warps + 1), pl.smem, st);
+    if (rc != 0) {
+      g_last_cuda = rc;
+      return MGS_ECUDA;
+    }
+    return MGS_OK;
   }
   mgs::Params pr{};
   pr.A = A;

@@ -3,6 +3,7 @@
 // the CPU.  The host intrinsics are correctly rounded like the GPU's, so the results are
 // the same bits.  Not used by the solver itself.
 #include "ddqd.cuh"
+#include "wide.cuh"
 
 namespace {
 
@@ -161,4 +162,76 @@ EXPORT void h_update_split_qd(const double* y, const double* c, const double* x,
     Q::pcombine(kFp, a, b);
     Q::pfinal(kFp, a, out + part * 4);
   }
+}
+
+// ------------------------------------------------------------------ wide.cuh (limbs in, limbs out)
+namespace {
+template <int L>
+struct W {
+  using N = mgs::Wide<L>;
+  mgs::u32 w[N::S];
+  explicit W(const double* v) { N::of_limbs(v, w); }
+  typename N::num num() const { return N::unpack(w); }
+};
+template <int L>
+void wide_update(const double* y, const double* c, const double* x, double* out) {
+  using N = mgs::Wide<L>;
+  mgs::u32 o[N::S];
+  const W<L> cr(c), ci(c + L), xr(x), xi(x + L);
+  N::update(W<L>(y).num(), cr.num(), xr.num(), ~0u, ci.num(), xi.num(), 0u, o);
+  N::to_limbs(o, out);
+  N::update(W<L>(y + L).num(), cr.num(), xi.num(), ~0u, ci.num(), xr.num(), ~0u, o);
+  N::to_limbs(o, out + L);
+}
+// re and im of sum conj(x) y, all terms at one exponent
+template <int L>
+void wide_dot(int n, const double* x, const double* y, double* out) {
+  using N = mgs::Wide<L>;
+  int E = -4 * N::BIAS;
+  for (int i = 0; i < n; ++i)
+    for (int p = 0; p < 4; ++p) {
+      const int e = W<L>(x + 2 * L * i + (p & 1) * L).num().e + W<L>(y + 2 * L * i + (p >> 1) * L).num().e;
+      E = e > E ? e : E;
+    }
+  E += N::SUMBITS;
+  typename N::sum re, im;
+  N::clear(re);
+  N::clear(im);
+  for (int i = 0; i < n; ++i) {
+    const W<L> xr(x + 2 * L * i), xi(x + 2 * L * i + L), yr(y + 2 * L * i), yi(y + 2 * L * i + L);
+    N::mac2(re, E, xr.num(), yr.num(), 0u, xi.num(), yi.num(), 0u);
+    N::mac(im, E, xr.num(), yi.num(), 0u);
+    N::mac(im, E, xi.num(), yr.num(), ~0u);
+  }
+  mgs::u32 o[N::S];
+  N::store(re, E, o);
+  N::to_limbs(o, out);
+  N::store(im, E, o);
+  N::to_limbs(o, out + L);
+}
+// op 0: v as it is, 1: v / d, 2: v d, 3: sqrt(v)
+template <int L>
+void wide_op(int op, const double* v, const double* d, double* out) {
+  using N = mgs::Wide<L>;
+  W<L> a(v);
+  mgs::u32 o[N::S];
+  for (int i = 0; i < N::S; ++i) o[i] = a.w[i];
+  if (op == 1) N::div_words(a.w, W<L>(d).w, o);
+  if (op == 2) N::mul_words(a.w, W<L>(d).w, o);
+  if (op == 3) N::sqrt_words(a.w, o);
+  N::to_limbs(o, out);
+}
+}  // namespace
+
+EXPORT void h_wide_update(int L, const double* y, const double* c, const double* x, double* out) {
+  L == 2 ? wide_update<2>(y, c, x, out) : wide_update<4>(y, c, x, out);
+}
+EXPORT void h_wide_dot(int L, int n, const double* x, const double* y, double* out) {
+  L == 2 ? wide_dot<2>(n, x, y, out) : wide_dot<4>(n, x, y, out);
+}
+EXPORT void h_wide_op(int L, int op, const double* v, const double* d, double* out) {
+  L == 2 ? wide_op<2>(op, v, d, out) : wide_op<4>(op, v, d, out);
+}
+EXPORT int h_wide_positive(int L, const double* v) {
+  return L == 2 ? mgs::Wide<2>::positive(W<2>(v).w) : mgs::Wide<4>::positive(W<4>(v).w);
 }

@@ -1,0 +1,665 @@
+// Single-system MGS least squares with whole columns per CTA and no grid-wide barrier during
+// the sweep (Section 3, Figure 1 and Eq. 1; Section 6), on the wide binary arithmetic of
+// wide.cuh.
+//
+// What bounds it: the chain of n dependent steps.  Pivot k must reach the owner of column
+// k+1, which projects, divides, updates and passes pivot k+1 on; the other columns of a step
+// are work for a microsecond or two beside it.  So the layout takes off that chain what it
+// can:
+//   * A CTA owns panels of `bw` consecutive columns (cyclic over the CTAs), all rows, in
+//     shared memory.  A column's Gram entry needs no other CTA: no partial sums in global
+//     memory and no barrier between CTAs in a step.
+//   * All warps of a CTA share its columns: a warp takes 16 rows of a column at a time, the
+//     real part in lanes 0..15 and the imaginary part in lanes 16..31 (the products of one
+//     part are a lane's own instruction stream, half as long as an element's).  One warp
+//     per column adds the warps' sums (integers: exact and independent of order) and divides.
+//     Column k+1 is taken first and by all warps.
+//   * One more warp receives pivots: it polls the pivot's flag and has the column copied into
+//     a ring of shared-memory stages by bulk copies (cp.async.bulk); the others wait on the
+//     stage's mbarrier.  A CTA that is behind finds its next pivots already there.
+//   * Published pivots travel in the caller's A (column k's own memory, as planes of 16-byte
+//     words; only its owner ever reads the input there), so a pivot needs no buffer that
+//     could be reused too early.  Q takes its place after the sweep.
+//   * Every CTA forms G_kk itself, in a third of its warps beside the dot products, so that
+//     nothing but the rows passes between CTAs.  (CTAs cut the rows differently, so their G_kk
+//     may differ in the last of 112 or 224 bits; the owner of column k+1 stores r_kk.)
+// Back substitution uses the coefficients c_kj = r_kj / r_kk themselves: R x = y divided by
+// r_kk row by row is the unit triangular system sum_j c_kj x_j = c_kn, so there is neither a
+// division nor a scaled copy of R.  One CTA runs it while the others write Q and R: a thread
+// keeps its rows as sums in shared memory, a link takes x_k off all of them and normalises
+// one, and the columns of coefficients arrive by bulk copies some links ahead.
+//
+// Every wait is bounded: after the time limit it records a timeout status and raises the
+// abort flag, and all later waits fall through.
+#pragma once
+
+#include "mgs_kernel.cuh"
+#include "wide.cuh"
+
+namespace mgs {
+
+struct ColParams {
+  double* A;
+  long long lda;
+  double* b;
+  double* R;  // nullptr: not wanted
+  long long ldr;
+  double* x;
+  double* z;
+  int m, n, nc, aug;
+  int Bc, bw, w;          // CTAs, consecutive columns, slots per CTA
+  int warps, stages;      // warps that work on columns, pivot stages
+  int first;              // column k+1 goes before a step's other columns
+  u32* C;              // coefficients c_kj, k < j, packed: (j (j - 1) / 2 + k) * 2 S words
+  u32* Rd;             // r_kk: nc * S words
+  unsigned* flags;     // kPublished once pivot k's rows are published: nc words
+  unsigned* sync;      // [0] barrier arrivals, [1] abort, [2] a non-finite input, [3] rank deficient
+  int* status;
+  long long timeout_ns;
+  const int* skip;
+  unsigned long long* trace;  // phase timestamps, (nc + 1) x grid x 8 (trace builds only)
+};
+
+constexpr int kColWarps = 15;                      // most warps that work on columns: with the receiver 4 per sub-partition, 128 registers a thread
+constexpr int kColThreads = 32 * (kColWarps + 1);  // and the receiving one
+
+constexpr unsigned kPublished = 16;                // > kColWarps: shares of the warps that publish add up to it
+
+__host__ __device__ inline size_t col_part_words(int L) { return L == 2 ? 6 : 10; }  // a sum and its exponent
+// shared memory after the stages and the tile: partial sums (two parts a warp), coefficients,
+// G_kk of the pivots before the own columns and of the last one, G_kk of this step, mbarriers
+__host__ __device__ inline size_t col_smem_bytes(int L, int m, int w, int stages) {
+  size_t v = (size_t)(w + stages) * m * 16 * L;
+  v += (size_t)kColWarps * 2 * col_part_words(L) * 4;
+  v += (size_t)kColWarps * 4 * L * 4 + (size_t)(w + 2) * 2 * L * 4;
+  v += (size_t)(2 * stages) * 8;
+  return v + 64;
+}
+// back substitution: the sums, x, and a ring of columns of coefficients
+constexpr int kColBS = 4;
+__host__ __device__ inline size_t col_backsub_bytes(int L, int n) {
+  return (size_t)n * 2 * (L == 2 ? 24 : 48) + (size_t)n * 16 * L + (size_t)kColBS * n * 16 * L + 8 * kColBS + 64;
+}
+
+// ------------------------------------------------------------------ PTX
+__device__ __forceinline__ u32 smem_addr(const void* p) { return (u32)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(u64* bar, u32 count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(u64* bar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(u64* bar, u32 bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ bool mbar_try(u64* bar, u32 parity) {
+  u32 ok;
+  asm volatile(
+      "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, u32 bytes, u64* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+
+// Bounded wait for a phase of an mbarrier; false after a timeout or an abort.
+__device__ __forceinline__ bool mbar_wait(const ColParams& pr, u64* bar, u32 parity) {
+  if (mbar_try(bar, parity)) return true;
+  const unsigned long long t0 = globaltimer();
+  unsigned spins = 0;
+  while (!mbar_try(bar, parity)) {
+    if ((++spins & 63u) == 0) {
+      if (ld_acquire_u32(&pr.sync[1])) return false;
+      if ((long long)(globaltimer() - t0) > pr.timeout_ns) {
+        set_status(pr.status, ST_ETIMEOUT);
+        atomicExch(&pr.sync[1], 1u);
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// ------------------------------------------------------------------ planes
+// A column in shared or published memory: uint4 plane q of row l at q * m + l; part p of an
+// element is planes p * L / 2 .. (L words of 16 bytes per element).
+template <int L>
+__device__ __forceinline__ typename Wide<L>::num ld_num(const uint4* col, int m, int l, int part) {
+  u32 w[2 * L];
+#pragma unroll
+  for (int q = 0; q < L / 2; ++q) {
+    const uint4 v = col[(size_t)(part * (L / 2) + q) * m + l];
+    w[4 * q] = v.x;
+    w[4 * q + 1] = v.y;
+    w[4 * q + 2] = v.z;
+    w[4 * q + 3] = v.w;
+  }
+  return Wide<L>::unpack(w);
+}
+template <int L>
+__device__ __forceinline__ void st_words(uint4* col, int m, int l, int part, const u32* w) {
+#pragma unroll
+  for (int q = 0; q < L / 2; ++q)
+    col[(size_t)(part * (L / 2) + q) * m + l] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+}
+// the larger biased exponent of an element's parts
+template <int L>
+__device__ __forceinline__ int ld_exp(const uint4* col, int m, int l) {
+  const u32* c = reinterpret_cast<const u32*>(col);
+  if (L == 2) {
+    const u32 a = c[4 * (size_t)l] & 0xffffu, b = c[4 * ((size_t)m + l)] & 0xffffu;
+    return (int)max(a, b);
+  }
+  return (int)max(c[4 * ((size_t)m + l) + 3], c[4 * ((size_t)3 * m + l) + 3]);
+}
+
+// Sum of a over groups of 2^LEVELS lanes (one exponent in each group), in every lane of it.
+template <int L, int LEVELS>
+__device__ __forceinline__ void lane_sum(typename Wide<L>::sum& s) {
+  constexpr int K = Wide<L>::K;
+#pragma unroll
+  for (int off = 1; off < (1 << LEVELS); off <<= 1) {
+    u32 t[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) t[q] = __shfl_xor_sync(0xffffffffu, s.a[q], off);
+    add_words<K>(s.a, t);
+  }
+}
+// a sum and its exponent in shared memory, and back
+template <int L>
+__device__ __forceinline__ void st_sum(u32* p, const typename Wide<L>::sum& s, int E) {
+#pragma unroll
+  for (int q = 0; q < Wide<L>::K; ++q) p[q] = s.a[q];
+  p[Wide<L>::K] = (u32)E;
+}
+
+template <int L>
+__global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr) {
+  using N = Wide<L>;
+  using num = typename N::num;
+  using sum = typename N::sum;
+  constexpr int S = N::S, K = N::K, E = 2 * L;
+  if (pr.skip && *pr.skip) return;  // uniform over the grid
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nthreads = blockDim.x;
+  const int c = blockIdx.x, Bc = pr.Bc, bw = pr.bw, m = pr.m, nc = pr.nc, w = pr.w;
+  const int NW = pr.warps, NS = pr.stages;
+  extern __shared__ __align__(16) unsigned char csm[];
+  const size_t colv = (size_t)L * m;  // uint4 per column
+  uint4* stage = reinterpret_cast<uint4*>(csm);
+  uint4* tile = stage + (size_t)NS * colv;
+  constexpr int PW = L == 2 ? 6 : 10;
+  u32* parts = reinterpret_cast<u32*>(tile + (size_t)w * colv);  // a warp's sums: 2 x PW
+  u32* coefs = parts + (size_t)kColWarps * 2 * PW;               // c_kj of the pass's columns: 2 S words each
+  u32* gown = coefs + (size_t)kColWarps * 2 * S;                 // G_kk of the pivot before own column s; [w]: the last
+  u32* gcur = gown + (size_t)(w + 1) * S;                        // G_kk of this step
+  u64* full = reinterpret_cast<u64*>(gcur + S);                  // rows of a stage have arrived
+  u64* empty = full + NS;                                        // all warps are done with it
+  auto col_of = [&](int s) { return ((s / bw) * Bc + c) * bw + s % bw; };
+  auto gcol = [&](int j) { return (j < pr.n) ? pr.A + (size_t)j * pr.lda * E : pr.b; };
+  int wc = 0;  // own columns
+  while (wc < w && col_of(wc) < nc) ++wc;
+  const int jlast = wc > 0 ? col_of(wc - 1) : 0;  // own columns ascend with the slot
+  unsigned epoch = 0;
+
+  if (tid == 0) {
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(full + i, 1);
+      mbar_init(empty + i, NW);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  // the input, limbs to words
+  {
+    bool bad = false;
+    for (int idx = tid; idx < wc * m * 2; idx += nthreads) {
+      const int part = idx & 1, rest = idx >> 1;
+      const int s = rest / m, l = rest % m;
+      const double2* src = reinterpret_cast<const double2*>(gcol(col_of(s)) + (size_t)l * E + part * L);
+      double v[L];
+#pragma unroll
+      for (int q = 0; q < L / 2; ++q) {
+        const double2 d = src[q];
+        v[2 * q] = d.x;
+        v[2 * q + 1] = d.y;
+      }
+#pragma unroll
+      for (int q = 0; q < L; ++q) bad |= !finite64(v[q]);
+      u32 o[S];
+      N::of_limbs(v, o);
+      st_words<L>(tile + (size_t)s * colv, m, l, part, o);
+    }
+    if (bad) atomicOr(&pr.sync[2], 1u);
+  }
+  __syncthreads();
+
+  if (warp < NW) {
+    const int part = lane >> 4, lr = lane & 15;
+    auto sync_warps = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(NW * 32) : "memory"); };
+    // columns before jpub are followed by some column of another CTA
+    const int jpub = Bc == 1 ? 0 : jlast == nc - 1 ? jlast - jlast % bw : nc - 1;
+    bool alive = true;
+    u32 st = 0, turn = 0;  // the stage of the next pivot received, and its phase
+    int s0 = 0, next = wc > 0 ? c * bw : nc;  // the first own column not yet a pivot, and its slot
+    const int kend = jlast == nc - 1 ? nc : jlast;  // the last column's owner ends with its norm
+    // columns and warps of the last pass; the shares of a column in dots and in updates
+    int pnb = -1, pnorm = -1, wpd = 1, cd = 0, sd = 0, wpu = 1, cu = 0, su = 0;
+    if (next == 0 && jpub > 0) {  // column 0 is a pivot as it is
+      uint4* pub = reinterpret_cast<uint4*>(gcol(0));
+      for (int i = tid; i < (int)colv; i += NW * 32) pub[i] = tile[i];
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(pr.flags),
+                     "r"(warp == 0 ? kPublished - (unsigned)(NW - 1) : 1u)
+                     : "memory");
+    }
+    for (int k = 0; k < kend; ++k) {
+      const bool mine = next == k;
+      const uint4* x;
+      sync_warps();  // the last step's updates, made by other warps perhaps
+      MGS_TR(k, 0);
+      if (mine) {
+        x = tile + (size_t)s0 * colv;
+        ++s0;
+        next = col_of(s0);
+      } else {
+        x = stage + (size_t)st * colv;
+        if (alive) alive = __all_sync(0xffffffffu, mbar_wait(pr, full + st, turn));
+      }
+      MGS_TR(k, 1);
+      const bool crit = s0 < wc && next == k + 1;  // column k + 1 is the next pivot
+      // passes over the own columns after k: column k + 1 alone first, then as many columns as
+      // there are warps.  The first pass also forms G_kk.
+      int sb = s0;
+      bool norm = true;
+      do {
+        int nb = min(NW - 1, wc - sb);
+        if (crit && norm && pr.first) nb = 1;
+        if (nb != pnb || (int)norm != pnorm) {
+          // a dot is two products a row and part, a norm one: the warps are shared 2 : 2 : .. : 1
+          pnb = nb;
+          pnorm = norm;
+          wpd = nb == 0 ? 1 : norm ? max(1, 2 * NW / (2 * nb + 1)) : NW / nb;
+          cd = warp / wpd;
+          sd = warp - cd * wpd;
+          wpu = nb == 0 ? 1 : NW / nb;
+          cu = warp / wpu;
+          su = warp - cu * wpu;
+        }
+        const int nw0 = nb * wpd;  // the first warp on the norm
+        {
+          sum a;
+          int Ex = 0;
+          N::clear(a);
+          if (cd < nb) {
+            const uint4* y = tile + (size_t)(sb + cd) * colv;
+            const int l0 = sd * 16 + lr, dl = wpd * 16;
+            int e = 0;
+            for (int l = l0; l < m; l += dl) e = max(e, ld_exp<L>(x, m, l) + ld_exp<L>(y, m, l));
+            Ex = __reduce_max_sync(0xffffffffu, e) - 2 * N::BIAS + N::SUMBITS;
+            for (int l = l0; l < m; l += dl)  // re: xr yr + xi yi, im: xr yi - xi yr
+              N::mac2(a, Ex, ld_num<L>(x, m, l, 0), ld_num<L>(y, m, l, part), 0u, ld_num<L>(x, m, l, 1),
+                      ld_num<L>(y, m, l, part ^ 1), (u32)-part);
+          } else if (norm) {
+            const int l0 = (warp - nw0) * 16 + lr, dl = (NW - nw0) * 16;
+            int e = 0;
+            for (int l = l0; l < m; l += dl) e = max(e, ld_exp<L>(x, m, l));
+            Ex = 2 * (__reduce_max_sync(0xffffffffu, e) - N::BIAS) + N::SUMBITS;
+            for (int l = l0; l < m; l += dl) {
+              const num v = ld_num<L>(x, m, l, part);
+              N::mac(a, Ex, v, v, 0u);
+            }
+          }
+          lane_sum<L, 4>(a);
+          if (lr == 0) st_sum<L>(parts + (size_t)(warp * 2 + part) * PW, a, Ex);
+        }
+        if (norm) MGS_TR(k, 2);
+        sync_warps();
+        if (norm) MGS_TR(k, 3);
+        // over the warps: G_kk by the last warp, G_kj by a column's first warp, which then
+        // divides: c_kj = G_kj / G_kk
+        const bool head = cd < nb && sd == 0;
+        num v;
+        {
+          const bool gw = norm && warp == NW - 1;
+          if (head || gw) {
+            // the last warp adds the sums of both parts of the norm's warps, a column's first
+            // warp those of one part in each half
+            const int at = gw ? nw0 * 2 + lane : (warp + lr) * 2 + part;
+            const bool have = gw ? lane < 2 * (NW - nw0) : lr < wpd;
+            sum a;
+            int e = -4 * N::BIAS;
+            N::clear(a);
+            if (have) {
+              const u32* p = parts + (size_t)at * PW;
+#pragma unroll
+              for (int i = 0; i < K; ++i) a.a[i] = p[i];
+              e = (int)p[K];
+            }
+            const int Ex = __reduce_max_sync(0xffffffffu, e);
+            N::shift_sum(a, Ex - e);
+            lane_sum<L, 4>(a);
+            u32 f;
+            if (gw) {
+              u32 t[K], g[S];
+#pragma unroll
+              for (int q = 0; q < K; ++q) t[q] = __shfl_xor_sync(0xffffffffu, a.a[q], 16);
+              add_words<K>(a.a, t);
+              N::store(a, Ex, g);
+              if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i < S; ++i) gcur[i] = g[i];
+                if (crit || k == nc - 1) {
+                  u32* go = gown + (size_t)(crit ? s0 : w) * S;
+#pragma unroll
+                  for (int i = 0; i < S; ++i) go[i] = g[i];
+                  if (!N::positive(g) && !(pr.aug && k == nc - 1)) atomicOr(&pr.sync[3], 1u);
+                }
+              }
+            } else {
+              v = N::normalize(a, Ex, f);
+            }
+          }
+        }
+        if (norm) sync_warps();
+        if (head) {
+          const int j = col_of(sb + cd);
+          u32 g[S], q[S], f;
+#pragma unroll
+          for (int i = 0; i < S; ++i) g[i] = gcur[i];
+          v = N::quotient(v, N::unpack(g), f);
+          N::pack(v, f, q);
+          if (lr == 0) {
+            const bool ok = N::positive(g);
+            u32* cs = coefs + (size_t)(cd * 2 + part) * S;
+            uint4* dst = reinterpret_cast<uint4*>(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S);
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+              q[i] = ok ? q[i] : 0u;
+              cs[i] = q[i];
+            }
+#pragma unroll
+            for (int i = 0; i < S / 4; ++i)
+              __stcg(dst + i, make_uint4(q[4 * i], q[4 * i + 1], q[4 * i + 2], q[4 * i + 3]));
+          }
+        }
+        if (norm) MGS_TR(k, 4);
+        sync_warps();
+        // a_j -= c_kj a_k, this warp's rows; the next pivot also goes to its memory in A
+        if (cu < nb) {
+          const int j = col_of(sb + cu);
+          uint4* y = tile + (size_t)(sb + cu) * colv;
+          uint4* pub = reinterpret_cast<uint4*>(gcol(j));
+          const bool glob = j == k + 1 && j < jpub;
+          const u32* cs = coefs + (size_t)(cu * 2) * S;
+          u32 g[S];
+#pragma unroll
+          for (int i = 0; i < S; ++i) g[i] = cs[i];
+          const num cr = N::unpack(g);
+#pragma unroll
+          for (int i = 0; i < S; ++i) g[i] = cs[S + i];
+          const num cim = N::unpack(g);
+          for (int l = su * 16 + lr; l < m; l += wpu * 16) {  // re: y - cr xr + ci xi, im: y - cr xi - ci xr
+            u32 o[S];
+            N::update(ld_num<L>(y, m, l, part), cr, ld_num<L>(x, m, l, part), ~0u, cim, ld_num<L>(x, m, l, part ^ 1),
+                      (u32)-part, o);
+            st_words<L>(y, m, l, part, o);
+            if (glob) st_words<L>(pub, m, l, part, o);
+          }
+          // the shares of the column's warps add up to kPublished (the release orders the rows
+          // of all lanes, which the warp barrier collects)
+          if (glob) {
+            __syncwarp();
+            if (lane == 0)
+              asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(pr.flags + j),
+                           "r"(su == 0 ? kPublished - (unsigned)(wpu - 1) : 1u)
+                           : "memory");
+          }
+        }
+        if (norm) MGS_TR(k, 5);
+        norm = false;
+        sb += nb;
+      } while (sb < wc);
+      MGS_TR(k, 6);
+      if (!mine) {
+        __syncwarp();
+        if (lane == 0 && alive) mbar_arrive(empty + st);
+        if (++st == (u32)NS) {
+          st = 0;
+          turn ^= 1u;
+        }
+      }
+    }
+    // r_kk of the pivots before the own columns, and of the last one
+    sync_warps();
+    for (int s = tid; s <= wc; s += NW * 32) {
+      const int k = s < wc ? col_of(s) - 1 : nc - 1;
+      if (k < 0 || (s == wc && jlast != nc - 1)) continue;
+      u32 g[S], r[S];
+#pragma unroll
+      for (int i = 0; i < S; ++i) {
+        g[i] = gown[(size_t)(s < wc ? s : w) * S + i];
+        r[i] = 0u;
+      }
+      if (N::positive(g)) N::sqrt_words(g, r);
+#pragma unroll
+      for (int i = 0; i < S; ++i) pr.Rd[(size_t)k * S + i] = r[i];
+    }
+  } else if (warp == NW && lane == 0) {
+    // the receiving thread
+    auto wait_word = [&](const unsigned* flag, unsigned want) {
+      if (ld_acquire_u32(flag) >= want) return true;
+      const unsigned long long t0 = globaltimer();
+      unsigned spins = 0;
+      while (ld_acquire_u32(flag) < want) {
+        if ((++spins & 63u) == 0) {
+          if (ld_acquire_u32(&pr.sync[1])) return false;
+          if ((long long)(globaltimer() - t0) > pr.timeout_ns) {
+            set_status(pr.status, ST_ETIMEOUT);
+            atomicExch(&pr.sync[1], 1u);
+            return false;
+          }
+        }
+      }
+      return true;
+    };
+    u32 got = 0;
+    int own = 0;
+    for (int k = 0; k < jlast; ++k) {
+      if (k == col_of(own)) {
+        ++own;
+        continue;
+      }
+      const u32 st = got % (u32)NS, turn = got / (u32)NS;
+      if (turn > 0 && !mbar_wait(pr, empty + st, (turn - 1) & 1u)) break;
+      if (!wait_word(pr.flags + k, kPublished)) break;
+      asm volatile("fence.proxy.async;" ::: "memory");
+      mbar_expect(full + st, (u32)(m * 16 * L));
+      bulk_load(stage + (size_t)st * colv, gcol(k), (u32)(m * 16 * L), full + st);
+      ++got;
+    }
+    // no copy may be in flight when the CTA goes on to reuse its shared memory or leaves
+    for (u32 i = got > (u32)NS ? got - NS : 0; i < got; ++i) {
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try(full + i % (u32)NS, (i / (u32)NS) & 1u))
+        if ((long long)(globaltimer() - t0) > pr.timeout_ns) break;
+    }
+  }
+  MGS_TR(nc, 0);
+  grid_barrier(pr, epoch);
+  MGS_TR(nc, 1);
+
+  // ---------------------------------------------------------------- after the sweep
+  if (c == 0 && tid == 0) {
+    if (ld_acquire_u32(&pr.sync[2]))
+      set_status(pr.status, ST_ENONFINITE);
+    else if (ld_acquire_u32(&pr.sync[3]))
+      set_status(pr.status, ST_ERANK);
+  }
+  auto ld_w = [&](const u32* p, u32* o) {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+    for (int i = 0; i < S / 4; ++i) {
+      const uint4 v = __ldcg(q + i);
+      o[4 * i] = v.x;
+      o[4 * i + 1] = v.y;
+      o[4 * i + 2] = v.z;
+      o[4 * i + 3] = v.w;
+    }
+  };
+  auto st_limbs = [&](double* p, const u32* o) {
+    double v[L];
+    N::to_limbs(o, v);
+    double2* q = reinterpret_cast<double2*>(p);
+#pragma unroll
+    for (int i = 0; i < L / 2; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
+  };
+  // Q, the residual, R, z of the own columns
+  auto outputs = [&](int first, int count) {  // by `count` threads from thread `first` on
+    const int t0 = tid - first;
+    for (int idx = t0; idx < wc * m * 2; idx += count) {
+      const int part = idx & 1, rest = idx >> 1;
+      const int s = rest / m, l = rest % m, j = col_of(s);
+      u32 a[S], r[S], o[S];
+      const uint4* col = tile + (size_t)s * colv;
+#pragma unroll
+      for (int q = 0; q < L / 2; ++q) {
+        const uint4 v = col[(size_t)(part * (L / 2) + q) * m + l];
+        a[4 * q] = v.x;
+        a[4 * q + 1] = v.y;
+        a[4 * q + 2] = v.z;
+        a[4 * q + 3] = v.w;
+      }
+      double* dst = gcol(j) + (size_t)l * E + part * L;
+      if (j < pr.n) {
+        ld_w(pr.Rd + (size_t)j * S, r);
+        if (!N::positive(r)) continue;
+        N::div_words(a, r, o);
+        st_limbs(dst, o);
+      } else {
+        // the residual; an entry that no projection changed is left as the caller wrote it
+        double v[L];
+#pragma unroll
+        for (int q = 0; q < L; ++q) v[q] = dst[q];
+        N::of_limbs(v, o);
+        bool same = true;
+#pragma unroll
+        for (int q = 0; q < S; ++q) same &= o[q] == a[q];
+        if (!same) st_limbs(dst, a);
+      }
+    }
+    if (pr.R)
+      for (int s = 0; s < wc; ++s) {
+        const int j = col_of(s);
+        if (j >= pr.n) break;
+        for (int idx = t0; idx < 2 * j + 2; idx += count) {
+          const int k = idx >> 1, part = idx & 1;
+          u32 a[S], r[S], o[S];
+          ld_w(pr.Rd + (size_t)k * S, r);
+          double* dst = pr.R + ((size_t)j * pr.ldr + k) * E + part * L;
+          if (k < j) {
+            ld_w(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S, a);
+            N::mul_words(a, r, o);
+            st_limbs(dst, o);
+          } else if (part == 0) {
+            st_limbs(dst, r);
+          } else {
+#pragma unroll
+            for (int q = 0; q < L; ++q) dst[q] = 0.0;
+          }
+        }
+      }
+    if (pr.aug && pr.z && jlast == nc - 1 && t0 == 0) {
+      u32 r[S];
+      ld_w(pr.Rd + (size_t)(nc - 1) * S, r);
+      st_limbs(pr.z, r);
+    }
+  };
+  outputs(0, nthreads);
+  MGS_TR(nc, 2);
+  if (!pr.aug || pr.x == nullptr || c != 0) return;
+
+  // ---------------------------------------------------------------- back substitution (CTA 0)
+  // x_k = c_kn - sum_{j > k} c_kj x_j.  Item i = 2 row + part.
+  const int n = pr.n;
+  constexpr int SW = L == 2 ? 6 : 12;                            // a sum and its exponent, padded
+  u32* ys = reinterpret_cast<u32*>(csm);                         // 2 n sums; the tile is no longer needed
+  u32* y = ys + (size_t)2 * n * SW;                              // x, stored form
+  uint4* ring = reinterpret_cast<uint4*>(y + (size_t)2 * n * S);  // column k of the coefficients in slot k % 4
+  u64* cfull = reinterpret_cast<u64*>(ring + (size_t)kColBS * n * L);
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 0; i < kColBS; ++i) mbar_init(cfull + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+  }
+  __syncthreads();
+  // column k (rows 0 .. k - 1), the i-th column from the end
+  auto fetch = [&](int k, int i) {
+    const u32 bytes = (u32)k * 16 * L;
+    mbar_expect(cfull + i % kColBS, bytes);
+    bulk_load(ring + (size_t)(i % kColBS) * n * L, pr.C + (size_t)k * (k - 1) / 2 * 2 * S, bytes, cfull + i % kColBS);
+  };
+  if (tid == 0)
+    for (int i = 0; i < kColBS && n - 1 - i > 0; ++i) fetch(n - 1 - i, i);
+  for (int i = tid; i < n * 2; i += nthreads) {
+    u32 v[S];
+    ld_w(pr.C + ((size_t)n * (n - 1) / 2) * 2 * S + (size_t)i * S, v);
+    if ((i >> 1) == n - 1) {
+#pragma unroll
+      for (int q = 0; q < S; ++q) y[(size_t)i * S + q] = v[q];
+    }
+    const num v0 = N::unpack(v);
+    sum a;
+    N::clear(a);
+    N::add(a, v0.e + 4, v0, 0u);
+    st_sum<L>(ys + (size_t)i * SW, a, v0.e + 4);
+  }
+  __syncthreads();
+  bool live = true;
+  for (int k = n - 1, i = 0; k > 0; --k, ++i) {
+    if (live) live = mbar_wait(pr, cfull + i % kColBS, (u32)(i / kColBS) & 1u);
+    const u32* col = reinterpret_cast<const u32*>(ring + (size_t)(i % kColBS) * n * L);
+    // the items from the pivot row up, so that the next unknown comes first
+    for (int it = 2 * k - 1 - tid; it >= 0; it -= nthreads) {
+      const int p = it & 1;
+      u32* ya = ys + (size_t)it * SW;
+      const u32* c2 = col + (size_t)(it >> 1) * 2 * S;
+      const num cr = N::unpack(c2), ci = N::unpack(c2 + S);
+      const num x1 = N::unpack(y + (size_t)(2 * k + p) * S), x2 = N::unpack(y + (size_t)(2 * k + (p ^ 1)) * S);
+      sum a;
+#pragma unroll
+      for (int q = 0; q < K; ++q) a.a[q] = ya[q];
+      int Ex = (int)ya[K];
+      // two products of less than 2^(need - 13) in each of at most 2^11 links: |a| < 2^(Ex - 1)
+      const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
+      if (need > Ex) {
+        N::shift_sum(a, need - Ex);
+        Ex = need;
+      }
+      N::mac2(a, Ex, cr, x1, ~0u, ci, x2, (u32)-p);
+      if ((it >> 1) == k - 1) {
+        N::store(a, Ex, y + (size_t)it * S);
+      } else {
+        st_sum<L>(ya, a, Ex);
+      }
+    }
+    __syncthreads();
+    if (tid == 0 && live && k - kColBS > 0) {
+      asm volatile("fence.proxy.async;" ::: "memory");
+      fetch(k - kColBS, i + kColBS);
+    }
+  }
+  for (int i = tid; i < n * 2; i += nthreads) st_limbs(pr.x + (size_t)i * L, y + (size_t)i * S);
+  MGS_TR(nc, 3);
+}
+
+}  // namespace mgs

@@ -122,7 +122,8 @@ __device__ __forceinline__ void set_status(int* status, int code) { atomicCAS(st
 // The last CTA to arrive learns it from its own atomic and does not poll; the others poll
 // the counter alone and look at the abort flag and the clock every 64 polls, so the
 // common path costs one memory round trip per poll.
-__device__ __forceinline__ void grid_barrier(const Params& pr, unsigned& epoch) {
+template <class P>
+__device__ __forceinline__ void grid_barrier(const P& pr, unsigned& epoch) {
   __syncthreads();
   if (threadIdx.x == 0) {
     ++epoch;

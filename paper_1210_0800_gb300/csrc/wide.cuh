@@ -1,0 +1,635 @@
+// Double-double and quad-double reals as wide binary floating-point numbers on the integer
+// pipe of sm_103a.
+//
+// Why: this GPU issues 2 FP64 lane-instructions per clock and SM, but 64 integer
+// multiply-adds (32 x 32 + 64 bits) and 64 integer adds, shifts and selects.  A
+// quad-double product in error-free transforms is 70 FP64 instructions (2240 clocks of one
+// warp's sub-partition); the same product on 224-bit integers is 28 multiply-adds and about
+// 60 other instructions.  So inside the kernels a real is a sign, an exponent and an integer
+// mantissa; limbs appear only where numbers enter and leave.
+//
+// A number is (-1)^s (m / 2^(32 W)) 2^e with an integer m of W words whose top bit is set:
+//   L = 2 (double-double): stored in 4 words with 112 significant bits and a 16-bit exponent;
+//   L = 4 (quad-double):   stored in 8 words with 224 significant bits and a 32-bit exponent;
+// i.e. in the bytes of the L limbs.  The top bit of the mantissa is implied and holds the
+// sign.  All-zero words are zero: they read as a number so small (2^-32768, 2^-2^20) that it
+// vanishes beside every number that limbs can hold, and results that small are stored as
+// zero, so zero needs no special case.
+//
+// Accuracy (one operation, relative to the largest term): products and sums are formed to
+// 2^-124 (L = 2) and 2^-219 (L = 4) and rounded to nearest at 112 and 224 bits, so a result
+// is off by at most 2^-111.9 and 2^-218; double-double and quad-double arithmetic, also that
+// of ddqd.cuh, has 2^-104 .. 2^-106 and 2^-208 .. 2^-212.  Exponents do not overflow or
+// underflow on the way.  Where a result has an exact representation (small integers, powers
+// of two, exact quotients) it is exact.
+#pragma once
+
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+
+#if !defined(__CUDACC__)
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#endif
+
+namespace mgs {
+
+using u32 = uint32_t;
+using u64 = unsigned long long;
+
+// ------------------------------------------------------------------ words
+__host__ __device__ __forceinline__ u32 shf_r(u32 lo, u32 hi, int s) {  // low word of (hi:lo) >> s, s in 0..31
+#if defined(__CUDA_ARCH__)
+  return __funnelshift_r(lo, hi, s);
+#else
+  return s ? (lo >> s) | (hi << (32 - s)) : lo;
+#endif
+}
+__host__ __device__ __forceinline__ u32 shf_l(u32 lo, u32 hi, int s) {  // high word of (hi:lo) << s, s in 0..31
+#if defined(__CUDA_ARCH__)
+  return __funnelshift_l(lo, hi, s);
+#else
+  return s ? (hi << s) | (lo >> (32 - s)) : hi;
+#endif
+}
+__host__ __device__ __forceinline__ int clz32(u32 v) {
+#if defined(__CUDA_ARCH__)
+  return __clz((int)v);
+#else
+  return v ? __builtin_clz(v) : 32;
+#endif
+}
+
+// a[0..n) += b[0..n) (^ neg) + (neg & 1): adds or, for neg = ~0, subtracts.
+template <int N>
+__host__ __device__ __forceinline__ void add_signed(u32* a, const u32* b, u32 neg) {
+#if defined(__CUDA_ARCH__)
+  u32 t;
+  asm volatile("add.cc.u32 %0, %1, %1;" : "=r"(t) : "r"(neg));  // carry = neg & 1
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("addc.cc.u32 %0, %0, %1;" : "+r"(a[i]) : "r"(b[i] ^ neg));
+#else
+  u64 c = neg & 1;
+  for (int i = 0; i < N; ++i) {
+    c += (u64)a[i] + (b[i] ^ neg);
+    a[i] = (u32)c;
+    c >>= 32;
+  }
+#endif
+}
+
+// a[0..n) += b[0..n)
+template <int N>
+__host__ __device__ __forceinline__ void add_words(u32* a, const u32* b) {
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (i == 0)
+      asm volatile("add.cc.u32 %0, %0, %1;" : "+r"(a[i]) : "r"(b[i]));
+    else if (i < N - 1)
+      asm volatile("addc.cc.u32 %0, %0, %1;" : "+r"(a[i]) : "r"(b[i]));
+    else
+      asm volatile("addc.u32 %0, %0, %1;" : "+r"(a[i]) : "r"(b[i]));
+  }
+#else
+  u64 c = 0;
+  for (int i = 0; i < N; ++i) {
+    c += (u64)a[i] + b[i];
+    a[i] = (u32)c;
+    c >>= 32;
+  }
+#endif
+}
+
+// acc[0..2n] += a * (b[0], b[2], b[4], ...), n factors, each product at words 2j, 2j + 1;
+// the carry out of the last goes to word 2n (CARRY) or is known to be zero.
+template <int N, bool CARRY>
+__host__ __device__ __forceinline__ void mad_row(u32* acc, const u32* b, u32 a) {
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    if (j == 0)
+      asm volatile("mad.lo.cc.u32 %0, %1, %2, %0;" : "+r"(acc[0]) : "r"(a), "r"(b[0]));
+    else
+      asm volatile("madc.lo.cc.u32 %0, %1, %2, %0;" : "+r"(acc[2 * j]) : "r"(a), "r"(b[2 * j]));
+    if (j == N - 1 && !CARRY)
+      asm volatile("madc.hi.u32 %0, %1, %2, %0;" : "+r"(acc[2 * j + 1]) : "r"(a), "r"(b[2 * j]));
+    else
+      asm volatile("madc.hi.cc.u32 %0, %1, %2, %0;" : "+r"(acc[2 * j + 1]) : "r"(a), "r"(b[2 * j]));
+  }
+  if (CARRY) asm volatile("addc.u32 %0, %0, 0;" : "+r"(acc[2 * N]));
+#else
+  u32 carry = 0;
+  for (int j = 0; j < N; ++j) {
+    const u64 lo = ((u64)acc[2 * j + 1] << 32) | acc[2 * j];
+    const u64 p = (u64)a * b[2 * j];
+    u64 s = lo + p;
+    u32 c = s < lo;
+    const u64 s2 = s + carry;
+    c += s2 < s;
+    acc[2 * j] = (u32)s2;
+    acc[2 * j + 1] = (u32)(s2 >> 32);
+    carry = c;
+  }
+  if (CARRY) acc[2 * N] += carry;
+#endif
+}
+
+template <int N, int I>
+struct RowOf {  // rows I .. N - 1 of the truncated product (see Wide::mul)
+  __host__ __device__ static __forceinline__ void run(u32* ev, u32* od, const u32* a, const u32* b) {
+    constexpr int ne = I / 2 + 1, no = (I + 1) / 2;
+    // even chain: products t = 0, 2, ... of row I at words t, t + 1; top word 2 ne - 1
+    mad_row<ne, (2 * ne <= N)>(ev, b + (N - 1 - I), a[I]);
+    if constexpr (no > 0) mad_row<no, (2 * no + 1 <= N)>(od + 1, b + (N - I), a[I]);
+    if constexpr (I + 1 < N) RowOf<N, I + 1>::run(ev, od, a, b);
+  }
+};
+
+template <int L_>
+struct Wide {
+  static constexpr int L = L_;
+  static_assert(L == 2 || L == 4, "double-double or quad-double");
+  static constexpr int W = L == 2 ? 4 : 7;   // mantissa words
+  static constexpr int K = W + 1;            // words of a product or a sum
+  static constexpr int S = 2 * L;            // stored words
+  static constexpr int BIAS = L == 2 ? 32768 : 1 << 20;
+  static constexpr int SUMBITS = 13;         // a sum may have up to 2^12 terms
+
+  struct num {
+    u32 m[W];
+    int e;
+    u32 s;  // 0 or ~0
+  };
+  // A sum: the two's complement integer a of K words stands for (a / 2^(32 K)) 2^E.
+  struct sum {
+    u32 a[K];
+  };
+
+  // ---------------------------------------------------------------- stored form
+  __host__ __device__ static __forceinline__ int biased_exp(const u32* w) {
+    return L == 2 ? (int)(w[0] & 0xffffu) : (int)w[S - 1];
+  }
+  __host__ __device__ static __forceinline__ num unpack(const u32* w) {
+    num r;
+    constexpr int T = L == 2 ? 3 : 6;  // word with the sign and the top of the mantissa
+#pragma unroll
+    for (int i = 0; i < W; ++i) r.m[i] = w[i];
+    if (L == 2) r.m[0] &= 0xffff0000u;
+    r.m[W - 1] |= 0x80000000u;
+    r.e = biased_exp(w) - BIAS;
+    r.s = (u32)((int)w[T] >> 31);
+    return r;
+  }
+  // Stores (m, f / 2^32 below it) rounded to nearest.
+  __host__ __device__ static __forceinline__ void pack(const num& v, u32 f, u32* w) {
+    u32 m[W], inc[W];
+    int e = v.e;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      m[i] = v.m[i];
+      inc[i] = 0;
+    }
+    inc[0] = L == 2 ? 0x8000u : f >> 31;
+    const u32 top = m[W - 1];
+    add_signed<W>(m, inc, 0u);
+    e += (m[W - 1] < top) ? 1 : 0;  // 0.111...1 rounded up to 1: the words are zero, the top bit implied
+    const bool tiny = e < -(BIAS / 2);
+    const u32 keep = tiny ? 0u : ~0u;
+    m[W - 1] = (m[W - 1] & 0x7fffffffu) | (v.s & 0x80000000u);
+    if (L == 2) m[0] = (m[0] & 0xffff0000u) | (u32)(e + BIAS);
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = m[i] & keep;
+    if (L == 4) w[S - 1] = (u32)(e + BIAS) & keep;
+  }
+
+  // ---------------------------------------------------------------- products and sums
+  // p = the top K words of a * b.  The words of weight below 2^(32 (W - 1)) are not formed:
+  // 2^-124 (W = 4), 2^-219 (W = 7) of the product.
+  __host__ __device__ static __forceinline__ void mul(const u32* a, const u32* b, u32* p) {
+    u32 ev[K + 1], od[K + 1];
+#pragma unroll
+    for (int i = 0; i <= K; ++i) ev[i] = od[i] = 0;
+    RowOf<W, 0>::run(ev, od, a, b);
+    p[0] = ev[0];
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+    for (int i = 1; i < K; ++i) {
+      if (i == 1)
+        asm volatile("add.cc.u32 %0, %1, %2;" : "=r"(p[i]) : "r"(ev[i]), "r"(od[i]));
+      else if (i < K - 1)
+        asm volatile("addc.cc.u32 %0, %1, %2;" : "=r"(p[i]) : "r"(ev[i]), "r"(od[i]));
+      else
+        asm volatile("addc.u32 %0, %1, %2;" : "=r"(p[i]) : "r"(ev[i]), "r"(od[i]));
+    }
+#else
+    u64 c = 0;
+    for (int i = 1; i < K; ++i) {
+      c += (u64)ev[i] + od[i];
+      p[i] = (u32)c;
+      c >>= 32;
+    }
+#endif
+  }
+  // p >>= s, `fill` coming in at the top: whole words (any s >= 0) ...
+  __host__ __device__ static __forceinline__ void shift_words(u32* p, int s, u32 fill = 0u) {
+    int ws = s >> 5;
+    ws = ws > K ? K : ws;
+#pragma unroll 1
+    for (; ws > 0; --ws) {
+#pragma unroll
+      for (int i = 0; i + 1 < K; ++i) p[i] = p[i + 1];
+      p[K - 1] = fill;
+    }
+  }
+  // ... and the rest, s mod 32.  Exponents of one row or column are mostly close, so the whole
+  // words are left to a branch that warps mostly skip; the callers put one branch around the
+  // whole-word shifts of all their terms, which leaves the products in one basic block, where
+  // they hide each other's latency.
+  __host__ __device__ static __forceinline__ void shift_bits(u32* p, int s, u32 fill = 0u) {
+    const int b = s & 31;
+#pragma unroll
+    for (int i = 0; i < K; ++i) p[i] = shf_r(p[i], i + 1 < K ? p[i + 1] : fill, b);
+  }
+  __host__ __device__ static __forceinline__ void shift_down(u32* p, int s, u32 fill = 0u) {
+    if (s >= 32) shift_words(p, s, fill);
+    shift_bits(p, s, fill);
+  }
+  __host__ __device__ static __forceinline__ void clear(sum& a) {
+#pragma unroll
+    for (int i = 0; i < K; ++i) a.a[i] = 0u;
+  }
+  // a += x y (neg = 0) or a -= x y (neg = ~0); E >= the product's exponent
+  __host__ __device__ static __forceinline__ void mac(sum& a, int E, const num& x, const num& y, u32 neg) {
+    u32 p[K];
+    mul(x.m, y.m, p);
+    shift_down(p, E - x.e - y.e);
+    add_signed<K>(a.a, p, neg ^ x.s ^ y.s);
+  }
+  // a += x1 y1 (+-) x2 y2, the signs as in mac
+  __host__ __device__ static __forceinline__ void mac2(sum& a, int E, const num& x1, const num& y1, u32 neg1,
+                                                       const num& x2, const num& y2, u32 neg2) {
+    u32 p[K], q[K];
+    mul(x1.m, y1.m, p);
+    mul(x2.m, y2.m, q);
+    const int s1 = E - x1.e - y1.e, s2 = E - x2.e - y2.e;
+    if ((s1 | s2) >= 32) {
+      shift_words(p, s1);
+      shift_words(q, s2);
+    }
+    shift_bits(p, s1);
+    shift_bits(q, s2);
+    add_signed<K>(a.a, p, neg1 ^ x1.s ^ y1.s);
+    add_signed<K>(a.a, q, neg2 ^ x2.s ^ y2.s);
+  }
+  // a += x or a -= x
+  __host__ __device__ static __forceinline__ void add(sum& a, int E, const num& x, u32 neg) {
+    u32 p[K];
+    p[0] = 0u;
+#pragma unroll
+    for (int i = 0; i < W; ++i) p[i + 1] = x.m[i];
+    shift_down(p, E - x.e);
+    add_signed<K>(a.a, p, neg ^ x.s);
+  }
+  // b shifted down arithmetically: the same sum at an exponent larger by s.  What vanishes
+  // altogether becomes 0 and not -1: a sum of products with zeros has a sign too.
+  __host__ __device__ static __forceinline__ void shift_sum(sum& b, int s) {
+    const u32 sign = (u32)((int)b.a[K - 1] >> 31);
+    shift_down(b.a, s, s >= 32 * K ? 0u : sign);
+  }
+  // The number a sum stands for, and the word below its mantissa.
+  __host__ __device__ static __forceinline__ num normalize(const sum& in, int E, u32& f) {
+    u32 a[K];
+    num r;
+    r.s = (u32)((int)in.a[K - 1] >> 31);
+    u32 z[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      a[i] = in.a[i] ^ r.s;
+      z[i] = 0u;
+    }
+    z[0] = r.s & 1u;
+    add_signed<K>(a, z, 0u);
+#pragma unroll 1
+    for (int it = 1; it < K && a[K - 1] == 0u; ++it) {  // rarely: the terms cancelled by a word or more
+#pragma unroll
+      for (int i = K - 1; i > 0; --i) a[i] = a[i - 1];
+      a[0] = 0u;
+      E -= 32;
+    }
+    const bool zero = a[K - 1] == 0u;
+    const int lz = zero ? 0 : clz32(a[K - 1]);
+#pragma unroll
+    for (int i = 0; i < W; ++i) r.m[i] = shf_l(a[i], a[i + 1], lz);
+    f = a[0] << lz;
+    r.e = zero ? -BIAS : E - lz;
+    return r;
+  }
+  __host__ __device__ static __forceinline__ void store(const sum& a, int E, u32* w) {
+    u32 f;
+    const num r = normalize(a, E, f);
+    pack(r, f, w);
+  }
+
+  // y + x1 y1 (+-) x2 y2 stored, the signs as in mac.  One part of y - c x is y - cr xr + ci xi
+  // (real) or y - cr xi - ci xr (imaginary).
+  __host__ __device__ static __forceinline__ void update(const num& y, const num& x1, const num& y1, u32 neg1,
+                                                         const num& x2, const num& y2, u32 neg2, u32* w) {
+    u32 p[K], q[K];
+    sum a;
+    mul(x1.m, y1.m, p);
+    mul(x2.m, y2.m, q);
+    const int e1 = x1.e + y1.e, e2 = x2.e + y2.e;
+    int E = e1 > e2 ? e1 : e2;
+    E = (y.e > E ? y.e : E) + 3;  // three terms < 2^(E - 3)
+    a.a[0] = 0u;
+#pragma unroll
+    for (int i = 0; i < W; ++i) a.a[i + 1] = y.m[i];
+    const int s0 = E - y.e, s1 = E - e1, s2 = E - e2;
+    if ((s0 | s1 | s2) >= 32) {
+      shift_words(a.a, s0);
+      shift_words(p, s1);
+      shift_words(q, s2);
+    }
+    shift_bits(a.a, s0);
+    shift_bits(p, s1);
+    shift_bits(q, s2);
+    // the sum up to y's sign, which the result takes back
+    add_signed<K>(a.a, p, neg1 ^ x1.s ^ y1.s ^ y.s);
+    add_signed<K>(a.a, q, neg2 ^ x2.s ^ y2.s ^ y.s);
+    u32 f;
+    num r = normalize(a, E, f);
+    r.s ^= y.s;
+    pack(r, f, w);
+  }
+
+  // ---------------------------------------------------------------- division, square root
+  // floor(2^63 / (d + 1)) for a word d with its top bit set, or up to 2 below it
+  __host__ __device__ static __forceinline__ u32 reciprocal(u32 d) {
+    const u64 d1 = (u64)d + 1;
+#if defined(__CUDA_ARCH__)
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rz(d)));
+    u64 x = (u64)__float2uint_rz(r * 0x1p62f) << 1;  // 2^63 / d to about 22 bits
+    long long err = (long long)((1ull << 63) - x * d1);
+    // one Newton correction x + x err / 2^63, then whole steps to an underestimate
+    x += (u64)(((err >> 18) * (long long)(x >> 3)) >> 42);
+    err = (long long)((1ull << 63) - x * d1);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (err < 0) {
+        --x;
+        err += (long long)d1;
+      }
+    if (err >= (long long)d1) ++x;
+    return x > 0xffffffffull ? 0xffffffffu : (u32)x;
+#else
+    const u64 x = (1ull << 63) / d1;
+    return x > 0xffffffffull ? 0xffffffffu : (u32)x;
+#endif
+  }
+  // Schoolbook long division n / d (mantissas in [1/2, 1)), 28 bits a digit.  A digit comes
+  // from the remainder's top word times an underestimate of 1/d: it is too small by less
+  // than 8, which the next digits carry (the remainder stays below 8 d).  The quotient is a
+  // sum with the exponent E; 28 guard bits make its rounding exact where the quotient is.
+  static constexpr int DIGITS = L == 2 ? 5 : 9;
+  __host__ __device__ static __forceinline__ void divide(const num& n, const num& d, sum& q, int& E) {
+    u32 r[K + 1], nd[W];  // remainder, W fraction words below an integer word; 2^(32 W) - d
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      r[i] = n.m[i];
+      nd[i] = 0u;
+    }
+    r[W] = r[W + 1] = 0u;
+    add_signed<W>(nd, d.m, ~0u);
+    const u32 v = reciprocal(d.m[W - 1]);
+    clear(q);
+#pragma unroll 1
+    for (int t = 0; t < DIGITS; ++t) {
+#pragma unroll
+      for (int i = W; i > 0; --i) r[i] = shf_l(r[i - 1], r[i], 28);
+      r[0] <<= 28;
+      const u32 g = (u32)(((u64)r[W] * v) >> 31);
+      // r - g d = r - g + g (1 - d)
+      r[W] -= g;
+      mad_row<(W + 1) / 2, (W % 2 == 0)>(r, nd, g);      // words 0, 2, 4, ..
+      mad_row<W / 2, (W % 2 == 1)>(r + 1, nd + 1, g);    // words 1, 3, 5, ..
+      u32 low[K];
+#pragma unroll
+      for (int i = K - 1; i > 0; --i) {
+        q.a[i] = shf_l(q.a[i - 1], q.a[i], 28);
+        low[i] = 0u;
+      }
+      q.a[0] <<= 28;
+      low[0] = g;
+      add_words<K>(q.a, low);
+    }
+    E = 32 * K - 28 * DIGITS + n.e - d.e;
+    if ((n.s ^ d.s) != 0u) {
+      sum t = q;
+      clear(q);
+      add_signed<K>(q.a, t.a, ~0u);
+    }
+  }
+  __host__ __device__ static __forceinline__ num quotient(const num& n, const num& d, u32& f) {
+    sum q;
+    int E;
+    divide(n, d, q, E);
+    return normalize(q, E, f);
+  }
+  // x / d stored (words to words)
+  __host__ __device__ static __forceinline__ void div_words(const u32* x, const u32* d, u32* w) {
+    u32 f;
+    const num q = quotient(unpack(x), unpack(d), f);
+    pack(q, f, w);
+  }
+  // x * y stored
+  __host__ __device__ static __forceinline__ void mul_words(const u32* x, const u32* y, u32* w) {
+    const num a = unpack(x), b = unpack(y);
+    sum t;
+    clear(t);
+    const int E = a.e + b.e + 1;
+    mac(t, E, a, b, 0u);
+    store(t, E, w);
+  }
+  // sqrt(x) for x > 0 by Newton's iteration r <- (r + x / r) / 2 from the root of the leading
+  // bits in double precision (53 bits -> 106 -> 212 -> 424)
+  __host__ __device__ static __forceinline__ void sqrt_words(const u32* x, u32* w) {
+    const num v = unpack(x);
+    // an even exponent: v = h 2^(2 t), h in [1/4, 1) as a double (the top 53 bits, truncated)
+    const int t = v.e >> 1, odd = v.e & 1;  // v.e = 2 t + odd
+    const u64 top = ((u64)v.m[W - 1] << 32) | v.m[W - 2];
+    const double h = (double)(top >> 11) * (odd ? 0x1p-52 : 0x1p-53);
+    const double s = std::sqrt(h);  // in [1/2, sqrt 2)
+    num r = of_double(s);
+    r.e += t;
+#pragma unroll 1
+    for (int it = 0; it < (L == 2 ? 2 : 3); ++it) {
+      sum q, a;
+      int E;
+      divide(v, r, q, E);
+      const int top_e = (E > r.e ? E : r.e) + 2;
+      shift_sum(q, top_e - E);
+      a = q;
+      add(a, top_e, r, 0u);
+      u32 f;
+      r = normalize(a, top_e - 1, f);
+      pack(r, f, w);
+      r = unpack(w);
+    }
+  }
+
+  // ---------------------------------------------------------------- limbs
+  __host__ __device__ static __forceinline__ num of_double(double d) {
+    u64 b;
+#if defined(__CUDA_ARCH__)
+    b = (u64)__double_as_longlong(d);
+#else
+    std::memcpy(&b, &d, sizeof b);
+#endif
+    num r;
+    const int ex = (int)(b >> 52) & 0x7ff;
+    u64 m = b & 0xfffffffffffffull;
+    int e = ex - 1022;
+    if (ex) {
+      m |= 1ull << 52;
+    } else {
+      e = -1021;
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) r.m[i] = 0u;
+    r.s = (u32)((long long)b >> 63);
+    if (m == 0) {
+      r.m[W - 1] = 0x80000000u;
+      r.e = -BIAS;
+      r.s = 0u;
+      return r;
+    }
+    m <<= 11;
+    while (!(m >> 63)) {  // subnormal
+      m <<= 1;
+      --e;
+    }
+    r.m[W - 1] = (u32)(m >> 32);
+    r.m[W - 2] = (u32)m;
+    r.e = e;
+    return r;
+  }
+  // The stored form of L limbs (any limbs: their exact sum, rounded).
+  __host__ __device__ static __forceinline__ void of_limbs(const double* v, u32* w) {
+    num t[L];
+    int E = -BIAS;
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      t[i] = of_double(v[i]);
+      E = t[i].e > E ? t[i].e : E;
+    }
+    E += 3;
+    sum a;
+    clear(a);
+#pragma unroll
+    for (int i = 0; i < L; ++i) add(a, E, t[i], 0u);
+    store(a, E, w);
+  }
+  __host__ __device__ static __forceinline__ double scaled(u64 h, int e, bool neg) {
+    // (-1)^neg (h / 2^53) 2^e, h in [2^52, 2^53]
+    if (h >> 53) {
+      h >>= 1;
+      ++e;
+    }
+    u64 b;
+    const int ex = e + 1022;
+    if (ex >= 2047) {
+      b = 0x7ffull << 52;
+    } else if (ex >= 1) {
+      b = ((u64)ex << 52) | (h & 0xfffffffffffffull);
+    } else {  // subnormal: round to nearest even
+      const int s = 1 - ex;
+      if (s > 54) {
+        b = 0;
+      } else {
+        b = h >> s;
+        const u64 rest = h & ((1ull << s) - 1), half = 1ull << (s - 1);
+        b += (rest > half || (rest == half && (b & 1))) ? 1 : 0;
+      }
+    }
+    b |= (u64)neg << 63;
+    double d;
+#if defined(__CUDA_ARCH__)
+    d = __longlong_as_double((long long)b);
+#else
+    std::memcpy(&d, &b, sizeof d);
+#endif
+    return d;
+  }
+  // L limbs, each the double nearest to what the limbs before it leave (ties to even); the last
+  // one is cut off at 53 bits instead: below 2^-105 (L = 2) and 2^-211 (L = 4) of the value,
+  // no more than an operation on limbs leaves.
+  __host__ __device__ static __forceinline__ void to_limbs(const u32* w, double* v) {
+    const num x = unpack(w);
+    u32 m[W];
+    int e = x.e;
+    bool neg = x.s != 0u;
+    bool zero = e <= -(BIAS / 2);
+#pragma unroll
+    for (int i = 0; i < W; ++i) m[i] = x.m[i];
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      if (zero) {
+        v[k] = 0.0;
+        continue;
+      }
+      const u64 top = ((u64)m[W - 1] << 32) | m[W - 2];
+      u64 h = top >> 11;
+      u32 low = 0u;
+#pragma unroll
+      for (int i = 0; i < W - 2; ++i) low |= m[i];
+      const u32 rest = m[W - 2] & 0x7ffu;
+      const bool up = k < L - 1 && (rest > 0x400u || (rest == 0x400u && (low != 0u || (h & 1))));
+      h += up ? 1 : 0;
+      v[k] = scaled(h, e, neg);
+      if (k == L - 1) break;
+      // what is left: the bits below h, or (rounded up) 2^11 words .. minus them, negated
+      u32 r[W];
+#pragma unroll
+      for (int i = 0; i < W; ++i) r[i] = m[i];
+      r[W - 1] = 0u;
+      r[W - 2] = rest;
+      if (up) {
+        u32 z[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+          z[i] = r[i];
+          r[i] = 0u;
+        }
+        r[W - 2] = 0x800u;
+        add_signed<W>(r, z, ~0u);
+        neg = !neg;
+      }
+      int shift = 0;
+#pragma unroll 1
+      for (int it = 0; it < W && r[W - 1] == 0u; ++it) {
+#pragma unroll
+        for (int i = W - 1; i > 0; --i) r[i] = r[i - 1];
+        r[0] = 0u;
+        shift += 32;
+      }
+      zero = r[W - 1] == 0u;
+      const int lz = zero ? 0 : clz32(r[W - 1]);
+#pragma unroll
+      for (int i = W - 1; i > 0; --i) m[i] = shf_l(r[i - 1], r[i], lz);
+      m[0] = r[0] << lz;
+      e -= shift + lz;
+    }
+  }
+  // 0 < x, and x neither underflows nor overflows as a double
+  __host__ __device__ static __forceinline__ bool positive(const u32* w) {
+    const int e = biased_exp(w) - BIAS;
+    const u32 s = w[L == 2 ? 3 : 6] >> 31;
+    return s == 0u && e >= -1073 && e <= 1024;
+  }
+};
+
+}  // namespace mgs

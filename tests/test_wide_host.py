@@ -1,0 +1,182 @@
+"""The kernels' wide binary arithmetic (csrc/wide.cuh, compiled for the host) against exact
+rationals: limbs in and out, the update y - c x, dot products, quotient, product, square
+root.  The bounds are what the header states: a result is off by at most 2^-111 (L = 2) or
+2^-217 (L = 4) of its largest term, less than double-double's 2^-104 and quad-double's
+2^-208, and a representable result is exact."""
+
+import ctypes
+from fractions import Fraction as F
+
+import numpy as np
+import pytest
+
+import pins
+from paper_1210_0800_gb300 import build, inputs
+
+dp = ctypes.POINTER(ctypes.c_double)
+BITS = {2: 111, 4: 217}
+# limbs: the last one is cut to its own 53 bits, one unit of at most 2^-105 (2^-211) of the value
+OUT = {2: F(1, 2 ** 105), 4: F(1, 2 ** 211)}
+
+
+@pytest.fixture(scope="module")
+def hl():
+    lib = ctypes.CDLL(build.build_host())
+    i = ctypes.c_int
+    lib.h_wide_update.argtypes = [i, dp, dp, dp, dp]
+    lib.h_wide_dot.argtypes = [i, i, dp, dp, dp]
+    lib.h_wide_op.argtypes = [i, i, dp, dp, dp]
+    lib.h_wide_positive.argtypes = [i, dp]
+    return lib
+
+
+def P(a):
+    a = np.ascontiguousarray(a, dtype=np.float64)
+    return a, a.ctypes.data_as(dp)
+
+
+def op(hl, L, code, v, d=None):
+    o = np.zeros(L)
+    v, vp = P(v)
+    d, dd = P(np.zeros(L) if d is None else d)
+    hl.h_wide_op(L, code, vp, dd, o.ctypes.data_as(dp))
+    return o
+
+
+def val(x):
+    return sum((F(float(v)) for v in np.ravel(x)), F(0))
+
+
+def reals(L, seed, count, spread=(-60, 60)):
+    return pins.rand_limbs(L, seed, count, spread).reshape(count, L)
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_limbs_round_trip(hl, L):
+    """Normalised limbs whose value fits the mantissa come back bit for bit (all but those
+    with gaps between limbs), others to the rounding; zero, one, powers of two, subnormals
+    and unnormalised limbs too."""
+    same = 0
+    vals = reals(L, 41, 400)
+    for v in vals:
+        o = op(hl, L, 0, v)
+        same += np.array_equal(o, v)
+        assert abs(val(o) - val(v)) <= abs(val(v)) * OUT[L]
+        assert o[0] == v[0]
+    assert same >= (300 if L == 2 else 200)
+    for lead in (0.0, 1.0, -1.0, 2.0 ** -1074, -3 * 2.0 ** -1060, 2.0 ** 1023, 1.7e308, 5e-310):
+        v = np.zeros(L)
+        v[0] = lead
+        assert np.array_equal(op(hl, L, 0, v), v)
+    v = np.zeros(L)
+    v[:2] = [1.0, -1.0]  # limbs that cancel
+    assert not op(hl, L, 0, v).any()
+    v[:2] = [2.0 ** -80, 1.0]  # not ordered
+    assert val(op(hl, L, 0, v)) == 1 + F(1, 2 ** 80)
+    for e in range(54, 70):  # ties between the first two limbs go to the even leading limb
+        v = np.zeros(L)
+        v[0], v[1] = 1.0 + 2.0 ** -52, 2.0 ** -e
+        assert np.array_equal(op(hl, L, 0, v), v)
+
+
+@pytest.mark.parametrize("L", [2, 4])
+@pytest.mark.parametrize("spread", [(-1, 1), (-20, 20), (-200, 200)])
+def test_update_vs_rationals(hl, L, spread):
+    yy, cc, xx = (pins.rand_limbs(L, s, 400, spread).reshape(200, 2, L) for s in (51, 52, 53))
+    for i, (y, c, x) in enumerate(zip(yy, cc, xx)):
+        if i % 4 == 3:  # cancellation: y nearly c x
+            cr, ci, xr, xi = val(c[0]), val(c[1]), val(x[0]), val(x[1])
+            for p, want in enumerate((cr * xr - ci * xi, cr * xi + ci * xr)):
+                rest = want
+                for k in range(L):
+                    y[p, k] = float(rest)
+                    rest -= F(float(y[p, k]))
+        o = np.zeros((2, L))
+        (y, yp), (c, cp), (x, xp) = P(y), P(c), P(x)
+        hl.h_wide_update(L, yp, cp, xp, o.ctypes.data_as(dp))
+        cr, ci, xr, xi = val(c[0]), val(c[1]), val(x[0]), val(x[1])
+        for p, terms in enumerate(((val(y[0]), -cr * xr, ci * xi), (val(y[1]), -cr * xi, -ci * xr))):
+            # inputs and products are rounded as well: a few units of the largest term
+            bound = max(map(abs, terms)) * F(8, 2 ** BITS[L]) + abs(sum(terms)) * OUT[L]
+            assert abs(val(o[p]) - sum(terms)) <= bound, (i, p)
+
+
+@pytest.mark.parametrize("L", [2, 4])
+@pytest.mark.parametrize("n,spread", [(1, (-3, 3)), (7, (-30, 30)), (64, (-1, 1)), (300, (-100, 100))])
+def test_dot_vs_rationals(hl, L, n, spread):
+    x, y = (pins.rand_limbs(L, s, 2 * n, spread).reshape(n, 2, L) for s in (61, 62))
+    o = np.zeros((2, L))
+    (x, xp), (y, yp) = P(x), P(y)
+    hl.h_wide_dot(L, n, xp, yp, o.ctypes.data_as(dp))
+    X = [(val(a[0]), val(a[1])) for a in x]
+    Y = [(val(a[0]), val(a[1])) for a in y]
+    for p in range(2):
+        if p == 0:
+            terms = [t for (a, b), (c, d) in zip(X, Y) for t in (a * c, b * d)]
+        else:
+            terms = [t for (a, b), (c, d) in zip(X, Y) for t in (a * d, -b * c)]
+        bound = sum(map(abs, terms)) * F(4, 2 ** BITS[L]) + abs(sum(terms)) * OUT[L]
+        assert abs(val(o[p]) - sum(terms)) <= bound
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_quotient_product_root(hl, L):
+    a, d = reals(L, 71, 300), reals(L, 72, 300)
+    for v, w in zip(a, d):
+        q = val(v) / val(w)
+        assert abs(val(op(hl, L, 1, v, w)) - q) <= abs(q) * (F(4, 2 ** BITS[L]) + OUT[L])
+        p = val(v) * val(w)
+        assert abs(val(op(hl, L, 2, v, w)) - p) <= abs(p) * (F(4, 2 ** BITS[L]) + OUT[L])
+        w = np.abs(w[0]) / w[0] * w  # positive
+        r = val(op(hl, L, 3, w))
+        assert abs(r * r - val(w)) <= val(w) * (F(8, 2 ** BITS[L]) + 2 * OUT[L])
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_exact_results_are_exact(hl, L):
+    """Small integers and powers of two: quotients, products, roots and updates without
+    rounding; the leading word of the divisor at both ends of its range."""
+    def r(v):
+        o = np.zeros(L)
+        o[0] = v
+        return o
+
+    ints = inputs.uniform_int(81, 400, 1, 2 ** 26 - 1)
+    for a, b in zip(ints[::2], ints[1::2]):
+        a, b = float(a), float(b)
+        assert val(op(hl, L, 1, r(a * b), r(b))) == F(a)
+        assert val(op(hl, L, 1, r(-a * b), r(a))) == -F(b)
+        assert val(op(hl, L, 2, r(a), r(b))) == F(a) * F(b)
+        assert val(op(hl, L, 3, r(a * a * 2.0 ** 40))) == F(a) * 2 ** 20
+    for top in (1.0, 2.0 - 2.0 ** -52, 1.0 + 2.0 ** -31, 2.0 - 2.0 ** -31, 2.0 - 2.0 ** -30):
+        for q in (1.0, 3.0, 2.0 - 2.0 ** -51):
+            assert val(op(hl, L, 1, np.array([v for v in (top * q,)] + [float(F(top) * F(q) - F(top * q))] + [0.0] * (L - 2)),
+                          r(top))) == F(q)
+    for e in (-1000, -7, 0, 1, 6, 900):
+        assert val(op(hl, L, 3, r(2.0 ** (e & ~1)))) == F(2) ** ((e & ~1) // 2)
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_positive_follows_the_double_range(hl, L):
+    for v, want in ((1.0, 1), (0.0, 0), (-1.0, 0), (2.0 ** -1074, 1), (1.7e308, 1), (np.inf, 0)):
+        a, ap = P(np.array([v] + [0.0] * (L - 1)))
+        assert hl.h_wide_positive(L, ap) == want, v
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_small_integers_stay_exact(hl, L):
+    """Updates and dot products of small integers, zeros of either sign among the factors, are
+    exact (a product with zero vanishes and leaves no unit in the last place)."""
+    v = inputs.uniform_int(82, 12 * 500, -9, 9).reshape(500, 12).astype(np.float64)
+    for r in v:
+        y, c, x, c2, x2 = (np.zeros((2, L)) for _ in range(5))
+        for a, k in ((y, 0), (c, 2), (x, 4), (c2, 6), (x2, 8)):
+            a[:, 0] = r[k:k + 2] * (r[10] > 0 or k != 4)
+        o = np.zeros((2, L))
+        hl.h_wide_update(L, P(y)[1], P(c)[1], P(x)[1], o.ctypes.data_as(dp))
+        z = complex(*y[:, 0]) - complex(*c[:, 0]) * complex(*x[:, 0])
+        assert o[0, 0] == z.real and o[1, 0] == z.imag and not o[:, 1:].any()
+        p, q = np.stack([c, c2]), np.stack([x, x2])
+        hl.h_wide_dot(L, 2, P(p)[1], P(q)[1], o.ctypes.data_as(dp))
+        z = sum(complex(*a[:, 0]).conjugate() * complex(*b[:, 0]) for a, b in ((c, x), (c2, x2)))
+        assert o[0, 0] == z.real and o[1, 0] == z.imag and not o[:, 1:].any()
