@@ -170,13 +170,15 @@ int ls_solve_qd(double* A, int lda, double* b, double* x, double* R, int ldr, do
  */
 typedef struct {
   int threads;     /* threads per CTA: 128 or 256 (0 = 256) */
-  int ctas_per_sm; /* resident CTAs per SM, 1..4 (0 = 1) */
-  int split;       /* CTAs per system, 1, 2 or 4 (0 = automatic: 2 or 4 when the batch is
-                      smaller than half or a quarter of the resident CTAs and every slice
-                      keeps 32 rows); the CTAs of a system form a thread-block cluster, each
-                      holds a slice of the rows, the slices' Gram partials are summed
-                      through distributed shared memory */
-  int chunks;      /* most lanes that share one (column, part) of a system's Gram row in a
+  int ctas_per_sm; /* resident CTAs per SM, 1..4 (0 = 1 for limbs 1, 2 for limbs 2 and 4) */
+  int split;       /* CTAs per system, 1, 2 or 4; they form a thread-block cluster.  limbs 1: each
+                      holds a slice of the rows, the slices' Gram partials are summed through
+                      distributed shared memory (0 = automatic: 2 or 4 when the batch is smaller
+                      than half or a quarter of the resident CTAs and every slice keeps 32 rows).
+                      limbs 2 and 4: the columns are dealt out to them (0 = automatic: while a
+                      cluster would get fewer than two systems and each CTA keeps 16 columns, or 8
+                      while CTAs would stay idle) */
+  int chunks;      /* limbs 1 (checked but without effect otherwise): most lanes that share one (column, part) of a system's Gram row in a
                       step, i.e. rows per lane = ceil(slice rows / chunks): 0 = as many as
                       the threads allow (fewest rows per lane, deepest reduction trees);
                       1..threads caps it (more columns per pass, shallower trees) */

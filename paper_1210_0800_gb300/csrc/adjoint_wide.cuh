@@ -1,0 +1,233 @@
+// Adjoint of the batched least squares in double-double and quad-double on the wide binary
+// arithmetic of wide.cuh (outputs and conventions of mgs_adjoint_kernel, batched_kernel.cuh):
+//   u = R^{-H} G, w = R^{-1} u, grad_b = Q u, grad_A = r w^H - grad_b x^H.
+//
+// Both triangular solves run on the unit triangle c_kj = r_kj / r_kk: R^H u = G is
+// C^H (D u) = G and R w = u is C w = D^{-1} u with D = diag(r_kk), so no link of their chains
+// divides.  c is formed once, in parallel, and kept with its transpose in the system's own
+// grad_A (n (n - 1) elements; grad_A is written last), which makes both solves read rows.
+// What bounds it: the two chains (n links of two products and a normalisation) and the
+// conversions between limbs and words; one CTA per system.
+#pragma once
+
+#include "batched_wide.cuh"
+
+namespace mgs {
+
+// Shared memory: the sums of a solve; u, w, x (n elements), r, grad_b (m), as words; r_kk.
+__host__ __device__ inline size_t adjoint_wide_smem_bytes(int L, int max_m, int max_n) {
+  return (size_t)max_n * 2 * (L == 2 ? 24 : 48) + (3 * (size_t)max_n + 2 * (size_t)max_m) * 16 * L +
+         (size_t)max_n * 8 * L + 64;
+}
+
+template <int L, int T>
+__global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
+  using N = Wide<L>;
+  using num = typename N::num;
+  using sum = typename N::sum;
+  constexpr int SW = N::S, K = N::K, E = 2 * L, Q4 = L / 2, YW = L == 2 ? 6 : 12;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ __align__(16) unsigned char asm_[];
+  u32* ys = reinterpret_cast<u32*>(asm_);      // 2 n sums
+  u32* uw = ys + (size_t)ap.max_n * 2 * YW;    // u
+  u32* ww = uw + (size_t)ap.max_n * 2 * SW;    // the solve's unknowns: D u, then w
+  u32* xw = ww + (size_t)ap.max_n * 2 * SW;    // x
+  u32* rw = xw + (size_t)ap.max_n * 2 * SW;    // residual
+  u32* gw = rw + (size_t)ap.max_m * 2 * SW;    // grad_b
+  u32* dw = gw + (size_t)ap.max_m * 2 * SW;    // r_kk
+  int* sflag = reinterpret_cast<int*>(dw + (size_t)ap.max_n * SW);
+  auto packed = [](int k, int j) { return (size_t)j * (j + 1) / 2 + k; };
+  auto ld_limbs = [&](const double* p, u32* o) {
+    double v[L];
+    const double2* q = reinterpret_cast<const double2*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) {
+      const double2 d = q[i];
+      v[2 * i] = d.x;
+      v[2 * i + 1] = d.y;
+    }
+    N::of_limbs(v, o);
+  };
+  auto st_limbs = [&](double* p, const u32* o) {
+    double v[L];
+    N::to_limbs(o, v);
+    double2* q = reinterpret_cast<double2*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
+  };
+  auto cp = [&](u32* d, const u32* s) {
+#pragma unroll
+    for (int i = 0; i < SW; ++i) d[i] = s[i];
+  };
+
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) {
+      sflag[0] = (int)atomicAdd(ap.counter, 1u);
+      sflag[1] = ST_OK;
+    }
+    __syncthreads();
+    const int qi = sflag[0];
+    if (qi >= ap.batch) break;
+    const int sys = ap.order ? ap.order[qi] : qi;
+    const int m = ap.m_arr[sys], n = ap.n_arr[sys];
+    if (n < 1 || m < n || m > ap.max_m || n > ap.max_n) {
+      if (tid == 0) ap.status[sys] = ST_EINVAL;
+      continue;
+    }
+    const double* Q = ap.Q + (size_t)ap.a_off[sys] * E;
+    const double* R = ap.R + (size_t)ap.r_off[sys] * E;
+    const double* xv = ap.x + (size_t)ap.x_off[sys] * E;
+    const double* rv = ap.r + (size_t)ap.b_off[sys] * E;
+    const double* Gv = ap.G + (size_t)ap.x_off[sys] * E;
+    double* gA = ap.gA + (size_t)ap.a_off[sys] * E;
+    double* gb = ap.gb + (size_t)ap.b_off[sys] * E;
+    u32* C = reinterpret_cast<u32*>(gA);  // c_kj at (k n + j) and (j n + k), k < j
+    for (int i = tid; i < n; i += T) {
+      u32 o[SW];
+      ld_limbs(R + packed(i, i) * E, o);
+      cp(dw + (size_t)i * SW, o);
+      if (!N::positive(o)) sflag[1] = ST_ERANK;
+    }
+    for (int i = tid; i < 2 * m; i += T) {
+      u32 o[SW];
+      ld_limbs(rv + (size_t)i * L, o);
+      cp(rw + (size_t)i * SW, o);
+    }
+    for (int i = tid; i < 2 * n; i += T) {
+      u32 o[SW];
+      ld_limbs(xv + (size_t)i * L, o);
+      cp(xw + (size_t)i * SW, o);
+      ld_limbs(Gv + (size_t)i * L, o);
+      if (i < 2) cp(ww + (size_t)i * SW, o);  // (D u)_0
+      const num v = N::unpack(o);
+      sum a;
+      N::clear(a);
+      N::add(a, v.e + 4, v, 0u);
+      st_sum<L>(ys + (size_t)i * YW, a, v.e + 4);
+    }
+    __syncthreads();
+    for (int idx = tid; idx < n * (n - 1); idx += T) {
+      const int p = idx & 1, pi = idx >> 1;
+      int j = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)pi)) * 0.5f);  // pi = j (j - 1) / 2 + k, k < j
+      while (j * (j - 1) / 2 > pi) --j;
+      while ((j + 1) * j / 2 <= pi) ++j;
+      const int k = pi - j * (j - 1) / 2;
+      u32 o[SW];
+      ld_limbs(R + packed(k, j) * E + p * L, o);
+      N::div_words(o, dw + (size_t)k * SW, o);
+      cp(C + ((size_t)k * n + j) * 2 * SW + p * SW, o);
+      cp(C + ((size_t)j * n + k) * 2 * SW + p * SW, o);
+    }
+    __syncthreads();
+    // Unit triangular solves: link k takes the unknown k off the rows on its far side (`up`: the
+    // rows below k, with c_jk; else those above, with conj c_kj) and normalises the next one.
+    auto solve = [&](bool up) {
+      for (int t = 0; t < n - 1; ++t) {
+        const int k = up ? n - 1 - t : t;
+        const int items = 2 * (n - 1 - t);
+        for (int i = tid; i < items; i += T) {  // the next unknown's row first
+          const int r = up ? k - 1 - (i >> 1) : k + 1 + (i >> 1), p = i & 1;
+          u32 c1[SW], c2[SW];
+          const u32* cc = C + ((size_t)k * n + r) * 2 * SW;
+          cp(c1, cc);
+          cp(c2, cc + SW);
+          u32* ya = ys + (size_t)(2 * r + p) * YW;
+          const num cr = N::unpack(c1), ci = N::unpack(c2);
+          const num x1 = N::unpack(ww + (size_t)(2 * k + p) * SW), x2 = N::unpack(ww + (size_t)(2 * k + (p ^ 1)) * SW);
+          sum a;
+#pragma unroll
+          for (int q = 0; q < K; ++q) a.a[q] = ya[q];
+          int Ex = (int)ya[K];
+          const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
+          if (need > Ex) {
+            N::shift_sum(a, need - Ex);
+            Ex = need;
+          }
+          // re: y - cr xr + ci xi, im: y - cr xi - ci xr; the conjugate turns the second sign
+          N::mac2(a, Ex, cr, x1, ~0u, ci, x2, (p != 0) == up ? ~0u : 0u);
+          if (i < 2)
+            N::store(a, Ex, ww + (size_t)(2 * r + p) * SW);
+          else
+            st_sum<L>(ya, a, Ex);
+        }
+        __syncthreads();
+      }
+    };
+    solve(false);
+    // u = D^{-1} (D u); the right-hand side of the second solve is D^{-1} u
+    for (int i = tid; i < 2 * n; i += T) {
+      u32 o[SW], d[SW];
+      const u32* dk = dw + (size_t)(i >> 1) * SW;
+      N::div_words(ww + (size_t)i * SW, dk, o);
+      cp(uw + (size_t)i * SW, o);
+      N::div_words(o, dk, d);
+      if ((i >> 1) == n - 1) cp(ww + (size_t)i * SW, d);
+      const num v = N::unpack(d);
+      sum a;
+      N::clear(a);
+      N::add(a, v.e + 4, v, 0u);
+      st_sum<L>(ys + (size_t)i * YW, a, v.e + 4);
+    }
+    __syncthreads();
+    solve(true);
+    // grad_b = Q u: half a warp per part of a row, 16 lanes share its terms; Q is converted once
+    // per element part
+    for (int i = warp; i < m; i += T / 32) {
+      const int p = lane >> 4;
+      sum a;
+      int Ex = -4 * N::BIAS;
+      N::clear(a);
+      for (int k0 = 0; k0 < n; k0 += 16) {
+        const int k = k0 + (lane & 15);
+        u32 o[SW], t[SW];
+#pragma unroll
+        for (int q = 0; q < SW; ++q) o[q] = 0u;
+        if (k < n) ld_limbs(Q + ((size_t)k * m + i) * E + p * L, o);
+#pragma unroll
+        for (int q = 0; q < SW; ++q) t[q] = __shfl_xor_sync(0xffffffffu, o[q], 16);
+        const u32* uk = uw + (size_t)min(k, n - 1) * 2 * SW;
+        // re: qr ur - qi ui, im: qi ur + qr ui (a zero Q past the last column adds nothing)
+        const num q1 = N::unpack(o), q2 = N::unpack(t), ur = N::unpack(uk), ui = N::unpack(uk + SW);
+        const int need = max(q1.e + ur.e, q2.e + ui.e) + N::SUMBITS;
+        if (need > Ex) {
+          N::shift_sum(a, need - Ex);
+          Ex = need;
+        }
+        N::mac2(a, Ex, q1, ur, 0u, q2, ui, p ? 0u : ~0u);
+      }
+      const int top = __reduce_max_sync(0xffffffffu, Ex);
+      N::shift_sum(a, top - Ex);
+      lane_sum<L, 4>(a);
+      u32 o[SW];
+      N::store(a, top, o);
+      if ((lane & 15) == 0) {
+        cp(gw + (size_t)(2 * i + p) * SW, o);
+        st_limbs(gb + (size_t)(2 * i + p) * L, o);
+      }
+    }
+    __syncthreads();
+    // grad_A, element (i, j): r_i conj(w_j) - g_i conj(x_j)
+    for (int t = tid; t < 2 * m * n; t += T) {
+      const int p = t & 1, rest = t >> 1;
+      const int j = rest / m, i = rest - j * m;
+      const num wr = N::unpack(ww + (size_t)2 * j * SW), wi = N::unpack(ww + (size_t)(2 * j + 1) * SW);
+      const num xr = N::unpack(xw + (size_t)2 * j * SW), xi = N::unpack(xw + (size_t)(2 * j + 1) * SW);
+      const num r1 = N::unpack(rw + (size_t)(2 * i + p) * SW), r2 = N::unpack(rw + (size_t)(2 * i + (p ^ 1)) * SW);
+      const num g1 = N::unpack(gw + (size_t)(2 * i + p) * SW), g2 = N::unpack(gw + (size_t)(2 * i + (p ^ 1)) * SW);
+      // re: wr rr + wi ri - xr gr - xi gi, im: wr ri - wi rr - xr gi + xi gr
+      const int Ex = max(max(wr.e + r1.e, wi.e + r2.e), max(xr.e + g1.e, xi.e + g2.e)) + 3;
+      sum a;
+      N::clear(a);
+      N::mac2(a, Ex, wr, r1, 0u, wi, r2, p ? ~0u : 0u);
+      N::mac2(a, Ex, xr, g1, ~0u, xi, g2, p ? 0u : ~0u);
+      u32 o[SW];
+      N::store(a, Ex, o);
+      st_limbs(gA + (size_t)t * L, o);
+    }
+    __syncthreads();
+    if (tid == 0) ap.status[sys] = sflag[1];
+  }
+}
+
+}  // namespace mgs

@@ -5,9 +5,16 @@
 
 #include "../../include/mgs_ddqd.h"
 #include "batched_kernel.cuh"
+#include "adjoint_wide.cuh"
+#include "batched_wide.cuh"
+#include "launch.cuh"
 
 namespace mgs {
 void set_last_cuda_error(int code);
+const void* batched_kernel_dd(int T, int S);
+const void* batched_kernel_qd(int T, int S);
+const void* adjoint_kernel_dd(int T);
+const void* adjoint_kernel_qd(int T);
 }
 
 namespace {
@@ -24,64 +31,79 @@ bool make_bplan(int L, int batch, int max_m, int max_n, const mgs_tune* tune, BP
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+  const bool wide = L != 1;  // double-double and quad-double: integer arithmetic (batched_wide.cuh)
   bp.T = (tune && tune->threads) ? tune->threads : 256;
-  bp.per_sm = (tune && tune->ctas_per_sm) ? tune->ctas_per_sm : 1;
+  bp.per_sm = (tune && tune->ctas_per_sm) ? tune->ctas_per_sm : wide ? 2 : 1;
   if (bp.T != 128 && bp.T != 256) return false;
   if (bp.per_sm < 1 || bp.per_sm > 4) return false;
   bp.cmax = tune ? tune->chunks : 0;
   if (bp.cmax < 0 || bp.cmax > bp.T) return false;
-  // systems split over S CTAs when the batch is smaller than the GPU (each slice keeps at
-  // least 32 rows); automatic unless the tuning asks for a split
+  // systems split over S CTAs; automatic unless the tuning asks for a split
   if (tune && tune->split) {
     bp.S = tune->split;
     if (bp.S != 1 && bp.S != 2 && bp.S != 4) return false;
+  } else if (wide) {
+    // Split while a resident cluster would get fewer than two systems (its largest one is then
+    // the launch's tail) and each CTA keeps 16 columns, or 8 while CTAs would stay idle.
+    // Double-double, ms at S = 1 / 2 / 4 with 304 resident CTAs: 512 systems of n <= 192 40 / 20.4 /
+    // 20.8, n <= 60 1.71 / 1.32 / 1.86, n <= 32 0.48 / 0.51 / 0.77; 1500 of n <= 64 4.1 / 5.2 / 7.2;
+    // 200 of n <= 120 7.5 / 5.1 / 3.3; 20 of n <= 40 0.51 / 0.38 / 0.29; 64 of n = 128 9.8 / 5.6 / 4.5
+    const long long slots = (long long)sms * bp.per_sm;
+    bp.S = 1;
+    while (bp.S < 4 && (long long)batch * bp.S < 2 * slots &&
+           max_n / (2 * bp.S) >= ((long long)batch * 2 * bp.S <= slots ? 8 : 16))
+      bp.S *= 2;
   } else {
+    // complex double: when the batch is smaller than the GPU and each slice keeps 32 rows
     bp.S = 1;
     while (bp.S < 4 && (long long)batch * 2 * bp.S <= (long long)sms * bp.per_sm && max_m / (2 * bp.S) >= 32)
       bp.S *= 2;
   }
-  bp.smem = mgs::batched_smem_bytes(L, bp.T, max_m, max_n, bp.S);
+  // the sizes that fit are those of the kernel with pivot, Gram row and reduction tree in
+  // shared memory, which the wide kernel's needs stay below
+  if (mgs::batched_smem_bytes(L, bp.T, max_m, max_n, bp.S) > 227 * 1024) return false;
+  bp.smem = wide ? mgs::batched_wide_smem_bytes(L, bp.T, max_m, max_n)
+                 : mgs::batched_smem_bytes(L, bp.T, max_m, max_n, bp.S);
   if (bp.smem > 227 * 1024) return false;
   const int clusters = (sms * bp.per_sm) / bp.S;
   bp.grid = bp.S * (clusters < batch ? clusters : batch);
-  bp.per_cta = mgs::batched_scratch_doubles(L, max_n);
+  bp.per_cta = wide ? mgs::batched_wide_scratch_doubles(L, max_n) : mgs::batched_scratch_doubles(L, max_n);
   bp.off_scr = 256;
   bp.total = bp.off_scr + sizeof(double) * (size_t)bp.per_cta * bp.grid;
   return true;
 }
 
-template <class Ar, int T, int S>
-int launch_batched_s(const mgs::BatchParams& p, const BPlan& pl, cudaStream_t st) {
-  auto kern = mgs::mgs_batched_kernel<Ar, T, S>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+template <int T>
+const void* batched_kernel_d(int S) {
+  return S == 4   ? (const void*)mgs::mgs_batched_kernel<mgs::D, T, 4>
+         : S == 2 ? (const void*)mgs::mgs_batched_kernel<mgs::D, T, 2>
+                  : (const void*)mgs::mgs_batched_kernel<mgs::D, T, 1>;
+}
+
+int launch_batched(int L, const mgs::BatchParams& p, const BPlan& pl, cudaStream_t st) {
+  const void* kern = L == 2   ? mgs::batched_kernel_dd(pl.T, pl.S)
+                     : L == 4 ? mgs::batched_kernel_qd(pl.T, pl.S)
+                     : pl.T == 128 ? batched_kernel_d<128>(pl.S)
+                                   : batched_kernel_d<256>(pl.S);
+  const cudaError_t e = mgs::ensure_smem(kern, pl.smem);
   if (e != cudaSuccess) return (int)e;
   mgs::BatchParams copy = p;
   void* args[] = {&copy};
-  if constexpr (S == 1) {
-    return (int)cudaLaunchKernel((const void*)kern, dim3(pl.grid), dim3(T), args, pl.smem, st);
-  } else {
-    // the clusters work independently (no CTA waits for another cluster)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(pl.grid);
-    cfg.blockDim = dim3(T);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = S;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return (int)cudaLaunchKernelExC(&cfg, (const void*)kern, args);
-  }
-}
-
-template <class Ar, int T>
-int launch_batched(const mgs::BatchParams& p, const BPlan& pl, cudaStream_t st) {
-  return pl.S == 4 ? launch_batched_s<Ar, T, 4>(p, pl, st)
-         : pl.S == 2 ? launch_batched_s<Ar, T, 2>(p, pl, st)
-                     : launch_batched_s<Ar, T, 1>(p, pl, st);
+  if (pl.S == 1) return (int)cudaLaunchKernel(kern, dim3(pl.grid), dim3(pl.T), args, pl.smem, st);
+  // the clusters work independently (no CTA waits for another cluster)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.grid);
+  cfg.blockDim = dim3(pl.T);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = pl.S;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return (int)cudaLaunchKernelExC(&cfg, kern, args);
 }
 
 int run_batched(int L, double* A, double* b, double* x, double* R, const int64_t* a_off, const int64_t* b_off,
@@ -130,13 +152,7 @@ int run_batched(int L, double* A, double* b, double* x, double* R, const int64_t
   p.cmax = pl.cmax;
   p.one = 1.0;
   p.nzero = -0.0;
-  int rc;
-  if (L == 1)
-    rc = (pl.T == 128) ? launch_batched<mgs::D, 128>(p, pl, st) : launch_batched<mgs::D, 256>(p, pl, st);
-  else if (L == 2)
-    rc = (pl.T == 128) ? launch_batched<mgs::DD, 128>(p, pl, st) : launch_batched<mgs::DD, 256>(p, pl, st);
-  else
-    rc = (pl.T == 128) ? launch_batched<mgs::QD, 128>(p, pl, st) : launch_batched<mgs::QD, 256>(p, pl, st);
+  const int rc = launch_batched(L, p, pl, st);
   if (rc != 0) {
     mgs::set_last_cuda_error(rc);
     return MGS_ECUDA;
@@ -144,14 +160,11 @@ int run_batched(int L, double* A, double* b, double* x, double* R, const int64_t
   return MGS_OK;
 }
 
-template <class Ar, int T>
-int launch_adjoint(const mgs::AdjParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto kern = mgs::mgs_adjoint_kernel<Ar, T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return (int)e;
-  mgs::AdjParams copy = p;
-  void* args[] = {&copy};
-  return (int)cudaLaunchKernel((const void*)kern, dim3(grid), dim3(T), args, smem, st);
+// The FP64 adjoint kernel, for systems whose vectors the wide one cannot hold in shared memory.
+const void* adjoint_kernel_large(int L, int T) {
+  if (L == 2)
+    return T == 128 ? (const void*)mgs::mgs_adjoint_kernel<mgs::DD, 128> : (const void*)mgs::mgs_adjoint_kernel<mgs::DD, 256>;
+  return T == 128 ? (const void*)mgs::mgs_adjoint_kernel<mgs::QD, 128> : (const void*)mgs::mgs_adjoint_kernel<mgs::QD, 256>;
 }
 
 int run_adjoint(int L, const double* Q, const double* R, const double* x, const double* r, const double* G, double* gA,
@@ -170,8 +183,13 @@ int run_adjoint(int L, const double* Q, const double* R, const double* x, const 
   const int T = (tune && tune->threads) ? tune->threads : 256;
   const int per_sm = (tune && tune->ctas_per_sm) ? tune->ctas_per_sm : 1;
   if ((T != 128 && T != 256) || per_sm < 1 || per_sm > 4) return MGS_EINVAL;
-  const size_t smem = mgs::adjoint_smem_bytes(L, max_n);
+  size_t smem = mgs::adjoint_smem_bytes(L, max_n);
   if (smem > 227 * 1024) return MGS_ENOSPACE;
+  // integer arithmetic where the vectors of a system (3 n + 2 m elements and n sums) fit, and
+  // grad_A, its scratch until it is written, is not Q
+  const size_t wide_smem = mgs::adjoint_wide_smem_bytes(L, max_m, max_n);
+  const bool wide = wide_smem <= 227 * 1024 && gA != Q;
+  if (wide) smem = wide_smem;
   if (ws_bytes < 256) return MGS_ENOSPACE;
   int grid = sms * per_sm;
   if (grid > batch) grid = batch;
@@ -203,11 +221,14 @@ int run_adjoint(int L, const double* Q, const double* R, const double* x, const 
   p.status = dev_status;
   p.one = 1.0;
   p.nzero = -0.0;
-  int rc;
-  if (L == 2)
-    rc = (T == 128) ? launch_adjoint<mgs::DD, 128>(p, grid, smem, st) : launch_adjoint<mgs::DD, 256>(p, grid, smem, st);
-  else
-    rc = (T == 128) ? launch_adjoint<mgs::QD, 128>(p, grid, smem, st) : launch_adjoint<mgs::QD, 256>(p, grid, smem, st);
+  const void* kern = !wide    ? adjoint_kernel_large(L, T)
+                     : L == 2 ? mgs::adjoint_kernel_dd(T)
+                              : mgs::adjoint_kernel_qd(T);
+  int rc = (int)mgs::ensure_smem(kern, smem);
+  if (rc == 0) {
+    void* args[] = {&p};
+    rc = (int)cudaLaunchKernel(kern, dim3(grid), dim3(T), args, smem, st);
+  }
   if (rc != 0) {
     mgs::set_last_cuda_error(rc);
     return MGS_ECUDA;

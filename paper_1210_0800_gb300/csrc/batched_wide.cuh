@@ -1,0 +1,409 @@
+// Batched least squares in double-double and quad-double on the wide binary arithmetic of
+// wide.cuh: the work queue, the method and the outputs of mgs_batched_kernel
+// (batched_kernel.cuh: Section 3, Figure 1 and Eq. 1; Section 6), organised for the integer
+// pipe.
+//
+// What bounds it: the integer multiply-adds of the products (a batch of hundreds of systems
+// fills the GPU), so no lane does what another lane has done:
+//   * A warp takes a trailing column through a whole step by itself -- dot product, division,
+//     update -- so a step has one barrier (the pivot's), and a warp reads its column twice
+//     in a row: the second time it is in L1.
+//   * A lane owns one part of a row: lanes 0..15 the real parts of 16 rows, lanes 16..31 the
+//     imaginary parts.  The 32 lanes read 16 consecutive elements.
+//   * The pivot is staged in shared memory as planes of 16-byte words, its norm summed from
+//     the staging threads' own words.
+//   * The system is kept in its own memory as words (the bytes of the limbs): converted where
+//     the input is checked, converted back where Q is formed.
+// Split systems (S = 2 or 4 CTAs of a cluster): the columns are dealt out to the CTAs, which
+// meet once per step; only the pivot column is read by all of them.
+#pragma once
+
+#include "batched_kernel.cuh"
+#include "mgs_column.cuh"
+
+namespace mgs {
+
+// Bytes of the back substitution's sums and unknowns.
+__host__ __device__ inline size_t batched_backsub_bytes(int L, int max_n) {
+  return (size_t)max_n * (2 * (L == 2 ? 24 : 48) + 16 * L);
+}
+// The largest back substitution kept in shared memory: two CTAs still fit an SM.  Larger ones
+// keep their sums in the global scratch.
+constexpr size_t kBatchedBacksubSmem = 64 * 1024;
+
+// Shared memory of one CTA: the pivot's planes, or the sums and x of the back substitution;
+// partial norms, the step's norm, flags.
+__host__ __device__ inline size_t batched_wide_body(int L, int max_m, int max_n) {
+  const size_t piv = (size_t)max_m * 16 * L, bs = batched_backsub_bytes(L, max_n);
+  return bs <= kBatchedBacksubSmem && bs > piv ? bs : piv;
+}
+__host__ __device__ inline size_t batched_wide_smem_bytes(int L, int T, int max_m, int max_n) {
+  return batched_wide_body(L, max_m, max_n) + (size_t)(T / 32) * col_part_words(L) * 4 + 64;
+}
+// Global scratch (doubles) of one cluster: packed c_kj, y, G_kk, r_kk, back substitution.
+__host__ __device__ inline long long batched_wide_scratch_doubles(int L, int max_n) {
+  const long long e = 2 * (long long)L, nc = max_n + 1;
+  const long long v = (long long)max_n * (max_n + 1) / 2 * e + nc * e + 2 * nc * L +
+                      (long long)batched_backsub_bytes(L, max_n) / 8;
+  return (v + 31) / 32 * 32;
+}
+
+template <int L, int T, int S>
+__global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParams bp) {
+  namespace cg = cooperative_groups;
+  using N = Wide<L>;
+  using num = typename N::num;
+  using sum = typename N::sum;
+  constexpr int SW = N::S, K = N::K, E = 2 * L, Q4 = L / 2, NW = T / 32;
+  constexpr int PW = L == 2 ? 6 : 10, YW = L == 2 ? 6 : 12;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int part = lane >> 4, lr = lane & 15;
+  const int rank = (int)(blockIdx.x % S);
+  const bool lead = rank == 0;
+  extern __shared__ __align__(16) unsigned char bsm[];
+  const size_t body = batched_wide_body(L, bp.max_m, bp.max_n);
+  const bool bs_smem = batched_backsub_bytes(L, bp.max_n) <= kBatchedBacksubSmem;
+  uint4* piv = reinterpret_cast<uint4*>(bsm);
+  u32* parts = reinterpret_cast<u32*>(bsm + body);
+  int* sflag = reinterpret_cast<int*>(parts + (size_t)NW * PW);
+  auto csync = [&]() {
+    if constexpr (S > 1)
+      cg::this_cluster().sync();
+    else
+      __syncthreads();
+  };
+  // the cluster's scratch: packed c_kj (k < j) at (j (j + 1) / 2 + k), y, G_kk, r_kk, as words
+  u32* scr = reinterpret_cast<u32*>(bp.ws + (size_t)(blockIdx.x / S) * bp.per_cta);
+  u32* Rp = scr;
+  u32* Yv = Rp + (size_t)bp.max_n * (bp.max_n + 1) / 2 * 2 * SW;
+  u32* Gd = Yv + (size_t)(bp.max_n + 1) * 2 * SW;
+  u32* Rd = Gd + (size_t)(bp.max_n + 1) * SW;
+  auto packed = [](int k, int j) { return (size_t)j * (j + 1) / 2 + k; };
+  auto ld_part = [&](const u32* p, u32* o) {  // one part's words
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) {
+      const uint4 v = q[i];
+      o[4 * i] = v.x;
+      o[4 * i + 1] = v.y;
+      o[4 * i + 2] = v.z;
+      o[4 * i + 3] = v.w;
+    }
+  };
+  auto ld_part_cg = [&](const u32* p, u32* o) {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) {
+      const uint4 v = __ldcg(q + i);
+      o[4 * i] = v.x;
+      o[4 * i + 1] = v.y;
+      o[4 * i + 2] = v.z;
+      o[4 * i + 3] = v.w;
+    }
+  };
+  auto st_part = [&](u32* p, const u32* o) {
+    uint4* q = reinterpret_cast<uint4*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) q[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+  };
+  auto st_limbs = [&](double* p, const u32* o) {
+    double v[L];
+    N::to_limbs(o, v);
+    double2* q = reinterpret_cast<double2*>(p);
+#pragma unroll
+    for (int i = 0; i < Q4; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
+  };
+
+  for (;;) {
+    csync();  // the cluster is done with the previous system
+    if (tid == 0) {
+      if (lead) sflag[0] = (int)atomicAdd(bp.counter, 1u);
+      sflag[1] = ST_OK;
+    }
+    csync();
+    int qi;
+    if constexpr (S > 1) {
+      qi = *cg::this_cluster().map_shared_rank(sflag, 0);
+      csync();  // no CTA leaves while a peer still reads rank 0's shared memory
+    } else {
+      qi = sflag[0];
+    }
+    if (qi >= bp.batch) break;
+    const int sys = bp.order ? bp.order[qi] : qi;
+    const int m = bp.m_arr[sys], n = bp.n_arr[sys];
+    if (n < 1 || m < n || m > bp.max_m || n > bp.max_n) {
+      if (tid == 0) bp.status[sys] = ST_EINVAL;
+      continue;
+    }
+    const int nc = n + 1;
+    double* A = bp.A + (size_t)bp.a_off[sys] * E;
+    double* bv = bp.b + (size_t)bp.b_off[sys] * E;
+    double* xv = bp.x + (size_t)bp.x_off[sys] * E;
+    auto col = [&](int j) -> double* { return (j < n) ? A + (size_t)j * m * E : bv; };
+    auto colw = [&](int j) { return reinterpret_cast<u32*>(col(j)); };
+    // the input of the own columns: limbs to words in place, non-finite entries found
+    {
+      bool bad = false;
+      for (int j = rank; j < nc; j += S) {
+        double* cj = col(j);
+        for (int i = tid; i < m * 2; i += T) {
+          double v[L];
+          const double2* src = reinterpret_cast<const double2*>(cj + (size_t)i * L);
+#pragma unroll
+          for (int q = 0; q < Q4; ++q) {
+            const double2 d = src[q];
+            v[2 * q] = d.x;
+            v[2 * q + 1] = d.y;
+          }
+#pragma unroll
+          for (int q = 0; q < L; ++q) bad |= !finite64(v[q]);
+          u32 o[SW];
+          N::of_limbs(v, o);
+          st_part(reinterpret_cast<u32*>(cj + (size_t)i * L), o);
+        }
+      }
+      if (bad) sflag[1] = ST_ENONFINITE;
+    }
+    for (int k = 0; k < nc; ++k) {
+      csync();  // column k is final
+      // the pivot and its norm
+      {
+        const u32* ck = colw(k);
+        sum a;
+        int Ex = -4 * N::BIAS;
+        N::clear(a);
+        for (int i = tid; i < m * 2; i += T) {
+          u32 v[SW];
+          ld_part_cg(ck + (size_t)i * SW, v);
+          st_words<L>(piv, m, i >> 1, i & 1, v);
+          const num x = N::unpack(v);
+          const int need = 2 * x.e + N::SUMBITS;
+          if (need > Ex) {
+            N::shift_sum(a, need - Ex);
+            Ex = need;
+          }
+          N::mac(a, Ex, x, x, 0u);
+        }
+        const int top = __reduce_max_sync(0xffffffffu, Ex);
+        N::shift_sum(a, top - Ex);
+        lane_sum<L, 5>(a);
+        if (lane == 0) st_sum<L>(parts + (size_t)warp * PW, a, top);
+      }
+      __syncthreads();
+      u32 g[SW];
+      {
+        sum a;
+        int e = -4 * N::BIAS;
+        N::clear(a);
+        if (lr < NW) {
+          const u32* p = parts + (size_t)lr * PW;
+#pragma unroll
+          for (int q = 0; q < K; ++q) a.a[q] = p[q];
+          e = (int)p[K];
+        }
+        const int top = __reduce_max_sync(0xffffffffu, e);
+        N::shift_sum(a, top - e);
+        lane_sum<L, 4>(a);
+        N::store(a, top, g);
+      }
+      if (lead && tid == 0) st_part(Gd + (size_t)k * SW, g);
+      if (k == nc - 1) break;  // the right-hand side: z^2; its column is the residual
+      const bool ok = N::positive(g);
+      if (!ok && tid == 0) sflag[1] = (sflag[1] == ST_OK) ? ST_ERANK : sflag[1];
+      const num gn = N::unpack(g);
+      // column j > k: the own columns, one warp each
+      int j = k + 1 + ((rank - (k + 1)) % S + S) % S + warp * S;
+      for (; j < nc; j += NW * S) {
+        u32* cj = colw(j);
+        sum a;
+        int Ex = -4 * N::BIAS;
+        N::clear(a);
+        u32 v[SW], o[SW], vn[SW], on[SW];  // this piece's words, and the next one's, loaded ahead
+        {
+          const int l = min(lr, m - 1);
+          ld_part(cj + (size_t)(2 * l + part) * SW, vn);
+          ld_part(cj + (size_t)(2 * l + (part ^ 1)) * SW, on);
+        }
+        for (int l = lr; l < m; l += 16) {  // re: xr yr + xi yi, im: xr yi - xi yr
+#pragma unroll
+          for (int i = 0; i < SW; ++i) {
+            v[i] = vn[i];
+            o[i] = on[i];
+          }
+          const int ln = min(l + 16, m - 1);
+          ld_part(cj + (size_t)(2 * ln + part) * SW, vn);
+          ld_part(cj + (size_t)(2 * ln + (part ^ 1)) * SW, on);
+          const num y1 = N::unpack(v), y2 = N::unpack(o);
+          const num x1 = ld_num<L>(piv, m, l, 0), x2 = ld_num<L>(piv, m, l, 1);
+          const int need = max(x1.e + y1.e, x2.e + y2.e) + N::SUMBITS;
+          if (need > Ex) {
+            N::shift_sum(a, need - Ex);
+            Ex = need;
+          }
+          N::mac2(a, Ex, x1, y1, 0u, x2, y2, (u32)-part);
+        }
+        const int top = __reduce_max_sync(0xffffffffu, Ex);
+        N::shift_sum(a, top - Ex);
+        lane_sum<L, 4>(a);
+        u32 f, c1[SW], c2[SW];
+        N::pack(N::quotient(N::normalize(a, top, f), gn, f), f, c1);
+#pragma unroll
+        for (int i = 0; i < SW; ++i) c1[i] = ok ? c1[i] : 0u;
+        if (lr == 0) st_part(((j < n) ? Rp + packed(k, j) * 2 * SW : Yv + (size_t)k * 2 * SW) + part * SW, c1);
+#pragma unroll
+        for (int i = 0; i < SW; ++i) {
+          const u32 t = c1[i];
+          c1[i] = __shfl_sync(0xffffffffu, t, 0);
+          c2[i] = __shfl_sync(0xffffffffu, t, 16);
+        }
+        const num cr = N::unpack(c1), ci = N::unpack(c2);
+        {
+          const int l = min(lr, m - 1);
+          ld_part(cj + (size_t)(2 * l + part) * SW, vn);
+        }
+        for (int l = lr; l < m; l += 16) {  // re: y - cr xr + ci xi, im: y - cr xi - ci xr
+#pragma unroll
+          for (int i = 0; i < SW; ++i) v[i] = vn[i];
+          const int ln = min(l + 16, m - 1);
+          ld_part(cj + (size_t)(2 * ln + part) * SW, vn);
+          N::update(N::unpack(v), cr, ld_num<L>(piv, m, l, part), ~0u, ci, ld_num<L>(piv, m, l, part ^ 1), (u32)-part,
+                    v);
+          st_part(cj + (size_t)(2 * l + part) * SW, v);
+        }
+        __syncwarp();
+      }
+    }
+    // r_kk
+    if (lead) {
+      __syncthreads();
+      for (int k = tid; k < nc; k += T) {
+        u32 gk[SW], r[SW];
+        ld_part(Gd + (size_t)k * SW, gk);
+#pragma unroll
+        for (int i = 0; i < SW; ++i) r[i] = 0u;
+        if (N::positive(gk)) N::sqrt_words(gk, r);
+        st_part(Rd + (size_t)k * SW, r);
+      }
+    }
+    __threadfence();
+    csync();
+    // q_j = a_j / r_jj of the own columns; the last column (b) is the residual
+    for (int j = rank; j < nc; j += S) {
+      u32 r[SW];
+      ld_part_cg(Rd + (size_t)j * SW, r);
+      const bool q = j < n;
+      if (q && !N::positive(r)) continue;
+      double* cj = col(j);
+      for (int i = tid; i < m * 2; i += T) {
+        u32 v[SW];
+        ld_part(reinterpret_cast<u32*>(cj + (size_t)i * L), v);
+        if (q) N::div_words(v, r, v);
+        st_limbs(cj + (size_t)i * L, v);
+      }
+    }
+    // the rest is rank 0's: R, back substitution, x, status
+    if (!lead) continue;
+    if (bp.R) {
+      double* Ro = bp.R + (size_t)bp.r_off[sys] * E;
+      for (int idx = tid; idx < n * (n + 1); idx += T) {
+        const int p = idx & 1, pi = idx >> 1;
+        int j = (int)((sqrtf(1.0f + 8.0f * (float)pi) - 1.0f) * 0.5f);  // pi = j (j + 1) / 2 + k
+        while (j * (j + 1) / 2 > pi) --j;
+        while ((j + 1) * (j + 2) / 2 <= pi) ++j;
+        const int k = pi - j * (j + 1) / 2;
+        double* dst = Ro + packed(k, j) * E + p * L;
+        u32 r[SW], v[SW];
+        ld_part_cg(Rd + (size_t)k * SW, r);
+        if (k < j) {
+          ld_part_cg(Rp + packed(k, j) * 2 * SW + p * SW, v);
+          N::mul_words(v, r, v);
+          st_limbs(dst, v);
+        } else if (p == 0) {
+          st_limbs(dst, r);
+        } else {
+#pragma unroll
+          for (int q = 0; q < L; ++q) dst[q] = 0.0;
+        }
+      }
+    }
+    // x_k = c_kn - sum_{j > k} c_kj x_j (R x = y divided by r_kk row by row): a thread keeps its
+    // items (2 row + part) as sums, a link takes x_k off all of them and normalises one
+    u32* ys = bs_smem ? reinterpret_cast<u32*>(bsm) : Rd + (size_t)(bp.max_n + 1) * SW;
+    u32* xs = ys + (size_t)2 * bp.max_n * YW;
+    __syncthreads();
+    for (int i = tid; i < n * 2; i += T) {
+      u32 v[SW];
+      ld_part_cg(Yv + (size_t)i * SW, v);
+      if ((i >> 1) == n - 1) {
+#pragma unroll
+        for (int q = 0; q < SW; ++q) xs[(size_t)i * SW + q] = v[q];
+      }
+      const num v0 = N::unpack(v);
+      sum a;
+      N::clear(a);
+      N::add(a, v0.e + 4, v0, 0u);
+      st_sum<L>(ys + (size_t)i * YW, a, v0.e + 4);
+    }
+    u32 nr[SW], ni[SW];  // the next link's coefficients of this thread's first item
+    auto fetch = [&](int k) {
+      const int it = 2 * k - 1 - tid;
+      if (it >= 0) {
+        const u32* c2 = Rp + packed(it >> 1, k) * 2 * SW;
+        ld_part_cg(c2, nr);
+        ld_part_cg(c2 + SW, ni);
+      }
+    };
+    if (n > 1) fetch(n - 1);
+    __syncthreads();
+    for (int k = n - 1; k > 0; --k) {
+      u32 c1[SW], c2[SW];
+#pragma unroll
+      for (int i = 0; i < SW; ++i) {
+        c1[i] = nr[i];
+        c2[i] = ni[i];
+      }
+      if (k > 1) fetch(k - 1);
+      // the items from the pivot row up, so that the next unknown comes first
+      for (int it = 2 * k - 1 - tid; it >= 0; it -= T) {
+        const int p = it & 1;
+        u32* ya = ys + (size_t)it * YW;
+        const num cr = N::unpack(c1), ci = N::unpack(c2);
+        const num x1 = N::unpack(xs + (size_t)(2 * k + p) * SW), x2 = N::unpack(xs + (size_t)(2 * k + (p ^ 1)) * SW);
+        sum a;
+#pragma unroll
+        for (int q = 0; q < K; ++q) a.a[q] = ya[q];
+        int Ex = (int)ya[K];
+        // two products of less than 2^(need - 13) in each of at most 2^11 links: |a| < 2^(Ex - 1)
+        const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
+        if (need > Ex) {
+          N::shift_sum(a, need - Ex);
+          Ex = need;
+        }
+        N::mac2(a, Ex, cr, x1, ~0u, ci, x2, (u32)-p);
+        if ((it >> 1) == k - 1)
+          N::store(a, Ex, xs + (size_t)it * SW);
+        else
+          st_sum<L>(ya, a, Ex);
+        if (it >= T) {
+          const u32* cn = Rp + packed((it - T) >> 1, k) * 2 * SW;
+          ld_part_cg(cn, c1);
+          ld_part_cg(cn + SW, c2);
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = tid; i < n * 2; i += T) st_limbs(xv + (size_t)i * L, xs + (size_t)i * SW);
+    __syncthreads();
+    if (tid == 0) {
+      // the input check comes first: a non-finite entry in any column wins over the rank
+      // deficiency it causes (the other flags are the same in every CTA)
+      int stv = sflag[1];
+      if constexpr (S > 1)
+        for (int pr = 1; pr < S; ++pr)
+          if (*cg::this_cluster().map_shared_rank(sflag + 1, pr) == ST_ENONFINITE) stv = ST_ENONFINITE;
+      bp.status[sys] = stv;
+    }
+  }
+}
+
+}  // namespace mgs
