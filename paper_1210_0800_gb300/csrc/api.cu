@@ -28,6 +28,7 @@ int cluster_capacity(int L, int cl, int T, size_t smem) {
   return L == 1 ? cluster_capacity_d(cl, T, smem) : L == 2 ? cluster_capacity_dd(cl, T, smem) : cluster_capacity_qd(cl, T, smem);
 }
 int column_capacity(int L, int threads, size_t smem);
+int column_clusters(int L, int cl, int threads, size_t smem);
 int launch_column(int L, const ColParams& pr, int threads, size_t smem, cudaStream_t stream);
 int blocks_per_sm_d(int kind, int T, size_t smem);
 int blocks_per_sm_dd(int kind, int T, size_t smem);
@@ -52,8 +53,9 @@ struct Plan {
   int T;     // threads per CTA (128 or 256)
   size_t smem;
   size_t off_sync, off_gsync, off_flags, off_P, off_V, off_Y, off_R, off_G, off_T, total, zero_bytes;
-  // the column kernel (col != 0): panel width, warps on columns, pivot stages, column k+1 first
-  int col, bw, warps, stages, first;
+  // the column kernel (col != 0): panel width, warps on columns, pivot stages, column k+1 first,
+  // cluster size
+  int col, bw, warps, stages, first, CL;
   size_t off_C, off_Rd;
 };
 
@@ -179,23 +181,35 @@ void column_plan(Plan& pl) {
   if (L == 1 || m > 2048) return;
   const int sms = device_sms();
   int bw = 1, warps = mgs::kColWarps, stages = 4, first = 1;
-  int Bc = nc < sms ? nc : sms;
   const int halves = (m + 15) / 16;  // 16-row pieces of a column
-  if (Bc > (nc + bw - 1) / bw) Bc = (nc + bw - 1) / bw;
-  const int w = (nc + bw * Bc - 1) / (bw * Bc) * bw;
+  // clusters of 8 CTAs (7 of 8 pivots are pushed to their next owner) when they leave a CTA no
+  // more columns than CTAs on all SMs would own; else of 4 or 2, or none
+  // (measured, us with / without: n = 32 DD 128 / 145, 256 1413 / 1531, 320x256 QD 2253 / 2347; with
+  // more than two columns a CTA the other columns' work hides the hand-off and the SMs that
+  // clusters leave idle cost more: 512 QD 7710 / 7561)
+  const int w = (nc + sms - 1) / sms * bw;
+  int CL = w <= 2 ? 8 : 1;
   if (warps > halves * (w + 1)) warps = halves * (w + 1);  // a pass: w columns and the norm
-  size_t smem;
-  for (;; --stages) {
-    if (stages < 2) return;
-    smem = mgs::col_smem_bytes(L, m, w, stages);
-    const size_t bs = mgs::col_backsub_bytes(L, pl.n);
-    if (bs > smem) smem = bs;
-    if (smem <= kMaxSmem) break;
-  }
-  const size_t pad = cta_per_sm_smem(1);
-  if (pad > smem && pad <= kMaxSmem) smem = pad;
   const int threads = 32 * (warps + 1);
-  if (mgs::column_capacity(L, threads, smem) * sms < Bc) return;
+  size_t smem = 0;
+  int Bc = 0;
+  const int most = stages;
+  for (; CL >= 1; CL /= 2) {
+    for (stages = most; stages >= 2; --stages) {
+      smem = mgs::col_smem_bytes(L, m, w, stages, CL);
+      const size_t bs = mgs::col_backsub_bytes(L, pl.n);
+      if (bs > smem) smem = bs;
+      if (smem <= kMaxSmem) break;
+    }
+    if (stages < 2) continue;
+    const size_t pad = cta_per_sm_smem(1);
+    if (pad > smem && pad <= kMaxSmem) smem = pad;
+    const int cap = CL > 1 ? mgs::column_clusters(L, CL, threads, smem) * CL : mgs::column_capacity(L, threads, smem) * sms;
+    Bc = nc < sms ? nc : sms;
+    if (Bc > cap) Bc = cap;
+    if (Bc > 0 && (Bc + CL - 1) / CL * CL <= cap && (nc + Bc - 1) / Bc <= w) break;
+  }
+  if (CL < 1) return;
   pl.col = 1;
   pl.kind = 0;
   pl.Br = 1;
@@ -206,6 +220,7 @@ void column_plan(Plan& pl) {
   pl.warps = warps;
   pl.stages = stages;
   pl.first = first;
+  pl.CL = CL;
   pl.T = (nc + Bc - 1) / Bc >= 16 ? 256 : 128;
   pl.smem = smem;
   size_t off = 64;
@@ -219,7 +234,7 @@ void column_plan(Plan& pl) {
   off = align256(off + sizeof(double) * (size_t)nc * (nc - 1) / 2 * 2 * L);
 #if defined(MGS_TRACE) && MGS_TRACE
   pl.off_T = off;
-  off = align256(off + sizeof(unsigned long long) * 8 * (size_t)(nc + 1) * Bc);
+  off = align256(off + sizeof(unsigned long long) * 8 * (size_t)(nc + 1) * (Bc + CL));
 #endif
   if (off > pl.total) pl.total = off;
 }
@@ -308,6 +323,7 @@ int run(int L, double* A, int lda, double* b, double* x, double* R, int ldr, dou
     cp.warps = pl.warps;
     cp.stages = pl.stages;
     cp.first = pl.first;
+    cp.CL = pl.CL;
     cp.C = reinterpret_cast<mgs::u32*>(wb + pl.off_C);
     cp.Rd = reinterpret_cast<mgs::u32*>(wb + pl.off_Rd);
     cp.flags = reinterpret_cast<unsigned*>(wb + pl.off_flags);
@@ -415,7 +431,7 @@ __attribute__((visibility("default"))) int mgs_trace_layout(int limbs, int m, in
   if (!make_plan(limbs, m, n, with_rhs, pl)) return MGS_ENOSPACE;
   *offset = pl.off_T;
   *steps = pl.nc + 1;
-  *ctas = pl.Br * pl.Bc;
+  *ctas = pl.col ? (pl.Bc + pl.CL - 1) / pl.CL * pl.CL : pl.Br * pl.Bc;
   return MGS_OK;
 }
 #endif

@@ -72,14 +72,10 @@ int launch_kernel(const Params& pr, int grid, int T, size_t smem, cudaStream_t s
   return (int)cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(T), args, smem, stream);
 }
 
-// Cluster variant: clusters of `cl` CTAs (the row blocks of a column group).  Launched
-// cooperatively when the driver accepts cooperative cluster launches, otherwise as a plain
-// cluster launch (the plan has checked that every cluster can be resident at once).
-template <class Ar>
-int launch_cluster_kernel(const Params& pr, int grid, int cl, int T, size_t smem, cudaStream_t stream) {
-  const void* kern = cluster_kernel<Ar>(T);
-  cudaError_t e = ensure_smem(kern, smem);
-  if (e != cudaSuccess) return (int)e;
+// Launch of clusters of `cl` CTAs: cooperatively when the driver accepts cooperative cluster
+// launches, otherwise as a plain cluster launch (the plan has checked that every cluster can
+// be resident at once).
+inline int launch_clusters(const void* kern, void** args, int grid, int cl, int T, size_t smem, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(T);
@@ -93,10 +89,8 @@ int launch_cluster_kernel(const Params& pr, int grid, int cl, int T, size_t smem
   attrs[1].id = cudaLaunchAttributeCooperative;
   attrs[1].val.cooperative = 1;
   cfg.attrs = attrs;
-  Params copy = pr;
-  void* args[] = {&copy};
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  e = cudaStreamIsCapturing(stream, &cap);
+  cudaError_t e = cudaStreamIsCapturing(stream, &cap);
   if (e != cudaSuccess) return (int)e;
   if (cap != cudaStreamCaptureStatusNone) {
     // inside a capture a refused launch would invalidate the graph: no second try
@@ -111,6 +105,17 @@ int launch_cluster_kernel(const Params& pr, int grid, int cl, int T, size_t smem
     e = cudaLaunchKernelExC(&cfg, kern, args);
   }
   return (int)e;
+}
+
+// Cluster variant: clusters of `cl` CTAs (the row blocks of a column group).
+template <class Ar>
+int launch_cluster_kernel(const Params& pr, int grid, int cl, int T, size_t smem, cudaStream_t stream) {
+  const void* kern = cluster_kernel<Ar>(T);
+  const cudaError_t e = ensure_smem(kern, smem);
+  if (e != cudaSuccess) return (int)e;
+  Params copy = pr;
+  void* args[] = {&copy};
+  return launch_clusters(kern, args, grid, cl, T, smem, stream);
 }
 
 // How many clusters of `cl` CTAs with `smem` bytes each can be resident at once.

@@ -18,13 +18,38 @@ int column_capacity(int L, int threads, size_t smem) {
   return per_sm;
 }
 
+// How many clusters of `cl` CTAs can be resident at once.
+int column_clusters(int L, int cl, int threads, size_t smem) {
+  const void* kern = column_kernel(L);
+  if (ensure_smem(kern, smem) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cl);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = cl;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 int launch_column(int L, const ColParams& pr, int threads, size_t smem, cudaStream_t stream) {
   const void* kern = column_kernel(L);
   cudaError_t e = ensure_smem(kern, smem);
   if (e != cudaSuccess) return (int)e;
   ColParams copy = pr;
   void* args[] = {&copy};
-  return (int)cudaLaunchCooperativeKernel(kern, dim3(pr.Bc), dim3(threads), args, smem, stream);
+  const int grid = (pr.Bc + pr.CL - 1) / pr.CL * pr.CL;
+  if (pr.CL == 1) return (int)cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, stream);
+  return launch_clusters(kern, args, grid, pr.CL, threads, smem, stream);
 }
 
 }  // namespace mgs

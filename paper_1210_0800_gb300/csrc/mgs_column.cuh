@@ -14,7 +14,10 @@
 //     part are a lane's own instruction stream, half as long as an element's).  One warp
 //     per column adds the warps' sums (integers: exact and independent of order) and divides.
 //     Column k+1 is taken first and by all warps.
-//   * One more warp receives pivots: it polls the pivot's flag and has the column copied into
+//   * Consecutive columns lie in the CTAs of a thread-block cluster: the owner of column k+1
+//     also stores its rows straight into the shared memory of the next owner (st.async on an
+//     mbarrier), without a flag, a fence or a trip through L2.
+//   * One more warp receives the other pivots: it polls the pivot's flag and has the column copied into
 //     a ring of shared-memory stages by bulk copies (cp.async.bulk); the others wait on the
 //     stage's mbarrier.  A CTA that is behind finds its next pivots already there.
 //   * Published pivots travel in the caller's A (column k's own memory, as planes of 16-byte
@@ -33,6 +36,8 @@
 // abort flag, and all later waits fall through.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "mgs_kernel.cuh"
 #include "wide.cuh"
 
@@ -50,6 +55,7 @@ struct ColParams {
   int Bc, bw, w;          // CTAs, consecutive columns, slots per CTA
   int warps, stages;      // warps that work on columns, pivot stages
   int first;              // column k+1 goes before a step's other columns
+  int CL;                 // CTAs of a cluster (1: none)
   u32* C;              // coefficients c_kj, k < j, packed: (j (j - 1) / 2 + k) * 2 S words
   u32* Rd;             // r_kk: nc * S words
   unsigned* flags;     // kPublished once pivot k's rows are published: nc words
@@ -68,11 +74,11 @@ constexpr unsigned kPublished = 16;                // > kColWarps: shares of the
 __host__ __device__ inline size_t col_part_words(int L) { return L == 2 ? 6 : 10; }  // a sum and its exponent
 // shared memory after the stages and the tile: partial sums (two parts a warp), coefficients,
 // G_kk of the pivots before the own columns and of the last one, G_kk of this step, mbarriers
-__host__ __device__ inline size_t col_smem_bytes(int L, int m, int w, int stages) {
-  size_t v = (size_t)(w + stages) * m * 16 * L;
+__host__ __device__ inline size_t col_smem_bytes(int L, int m, int w, int stages, int CL) {
+  size_t v = (size_t)(w + stages + (CL > 1 ? 1 : 0)) * m * 16 * L;  // in clusters also the pushed pivot
   v += (size_t)kColWarps * 2 * col_part_words(L) * 4;
   v += (size_t)kColWarps * 4 * L * 4 + (size_t)(w + 2) * 2 * L * 4;
-  v += (size_t)(2 * stages) * 8;
+  v += (size_t)(2 * stages + 2) * 8;
   return v + 64;
 }
 // back substitution: the sums, x, and a ring of columns of coefficients
@@ -102,6 +108,29 @@ __device__ __forceinline__ bool mbar_try(u64* bar, u32 parity) {
       : "memory");
   return ok != 0;
 }
+__device__ __forceinline__ bool mbar_try_cluster(u64* bar, u32 parity) {
+  u32 ok;
+  asm volatile(
+      "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// the address of a peer's shared memory in the cluster
+__device__ __forceinline__ u32 peer_addr(const void* p, u32 rank) {
+  u32 a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void peer_arrive(u32 bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void push16(u32 dst, const u32* w, u32 bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst),
+               "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, u32 bytes, u64* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_addr(dst)),
@@ -110,11 +139,13 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, u32 bytes,
 }
 
 // Bounded wait for a phase of an mbarrier; false after a timeout or an abort.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(const ColParams& pr, u64* bar, u32 parity) {
-  if (mbar_try(bar, parity)) return true;
+  auto test = [&]() { return CLUSTER ? mbar_try_cluster(bar, parity) : mbar_try(bar, parity); };
+  if (test()) return true;
   const unsigned long long t0 = globaltimer();
   unsigned spins = 0;
-  while (!mbar_try(bar, parity)) {
+  while (!test()) {
     if ((++spins & 63u) == 0) {
       if (ld_acquire_u32(&pr.sync[1])) return false;
       if ((long long)(globaltimer() - t0) > pr.timeout_ns) {
@@ -194,7 +225,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   extern __shared__ __align__(16) unsigned char csm[];
   const size_t colv = (size_t)L * m;  // uint4 per column
   uint4* stage = reinterpret_cast<uint4*>(csm);
-  uint4* tile = stage + (size_t)NS * colv;
+  uint4* push = stage + (size_t)NS * colv;  // the pivot before an own column, from the CTA before
+  uint4* tile = push + (pr.CL > 1 ? colv : 0);
   constexpr int PW = L == 2 ? 6 : 10;
   u32* parts = reinterpret_cast<u32*>(tile + (size_t)w * colv);  // a warp's sums: 2 x PW
   u32* coefs = parts + (size_t)kColWarps * 2 * PW;               // c_kj of the pass's columns: 2 S words each
@@ -202,6 +234,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   u32* gcur = gown + (size_t)(w + 1) * S;                        // G_kk of this step
   u64* full = reinterpret_cast<u64*>(gcur + S);                  // rows of a stage have arrived
   u64* empty = full + NS;                                        // all warps are done with it
+  u64* pfull = empty + NS;                                       // a pushed pivot has arrived
+  u64* pempty = pfull + 1;                                       // the CTA after has used the one pushed to it
   auto col_of = [&](int s) { return ((s / bw) * Bc + c) * bw + s % bw; };
   auto gcol = [&](int j) { return (j < pr.n) ? pr.A + (size_t)j * pr.lda * E : pr.b; };
   int wc = 0;  // own columns
@@ -214,6 +248,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       mbar_init(full + i, 1);
       mbar_init(empty + i, NW);
     }
+    mbar_init(pfull, 1);
+    mbar_init(pempty, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -239,7 +275,13 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     }
     if (bad) atomicOr(&pr.sync[2], 1u);
   }
-  __syncthreads();
+  // pushes between neighbours of a cluster
+  const int crank = c % pr.CL;
+  const bool push_in = crank != 0, push_out = pr.CL > 1 && crank != pr.CL - 1;
+  if (pr.CL > 1)
+    cooperative_groups::this_cluster().sync();  // no push before the peer's mbarriers are set up
+  else
+    __syncthreads();
 
   if (warp < NW) {
     const int part = lane >> 4, lr = lane & 15;
@@ -248,13 +290,24 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     const int jpub = Bc == 1 ? 0 : jlast == nc - 1 ? jlast - jlast % bw : nc - 1;
     bool alive = true;
     u32 st = 0, turn = 0;  // the stage of the next pivot received, and its phase
+    u32 pturn = 0;         // the phase of the next pushed pivot
+    bool used = false;     // the last step's pivot was pushed: tell the CTA before that it may push again
+    int pushes = 0;        // pivots pushed to the CTA after
+    const u32 rused = push_in ? peer_addr(pempty, crank - 1) : 0u;
+    const u32 rpush = push_out ? peer_addr(push, crank + 1) : 0u, rbar = push_out ? peer_addr(pfull, crank + 1) : 0u;
     int s0 = 0, next = wc > 0 ? c * bw : nc;  // the first own column not yet a pivot, and its slot
-    const int kend = jlast == nc - 1 ? nc : jlast;  // the last column's owner ends with its norm
+    const int kend = wc == 0 ? 0 : jlast == nc - 1 ? nc : jlast;  // the last column's owner ends with its norm
     // columns and warps of the last pass; the shares of a column in dots and in updates
     int pnb = -1, pnorm = -1, wpd = 1, cd = 0, sd = 0, wpu = 1, cu = 0, su = 0;
     if (next == 0 && jpub > 0) {  // column 0 is a pivot as it is
       uint4* pub = reinterpret_cast<uint4*>(gcol(0));
-      for (int i = tid; i < (int)colv; i += NW * 32) pub[i] = tile[i];
+      for (int i = tid; i < (int)colv; i += NW * 32) {
+        const uint4 v = tile[i];
+        pub[i] = v;
+        const u32 o[4] = {v.x, v.y, v.z, v.w};
+        if (push_out) push16(rpush + 16u * i, o, rbar);
+      }
+      ++pushes;
       __syncwarp();
       if (lane == 0)
         asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(pr.flags),
@@ -263,13 +316,22 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     }
     for (int k = 0; k < kend; ++k) {
       const bool mine = next == k;
+      const bool pushed = push_in && s0 < wc && next == k + 1;
       const uint4* x;
       sync_warps();  // the last step's updates, made by other warps perhaps
+      if (used && tid == 0) peer_arrive(rused);
+      used = false;
       MGS_TR(k, 0);
       if (mine) {
         x = tile + (size_t)s0 * colv;
         ++s0;
         next = col_of(s0);
+      } else if (pushed) {
+        x = push;
+        if (tid == 0) mbar_expect(pfull, (u32)(colv * 16));
+        if (alive) alive = __all_sync(0xffffffffu, mbar_wait<true>(pr, pfull, pturn));
+        pturn ^= 1u;
+        used = true;
       } else {
         x = stage + (size_t)st * colv;
         if (alive) alive = __all_sync(0xffffffffu, mbar_wait(pr, full + st, turn));
@@ -399,6 +461,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
           uint4* y = tile + (size_t)(sb + cu) * colv;
           uint4* pub = reinterpret_cast<uint4*>(gcol(j));
           const bool glob = j == k + 1 && j < jpub;
+          if (glob && push_out && pushes > 0 && alive)
+            alive = __all_sync(0xffffffffu, mbar_wait<true>(pr, pempty, (u32)(pushes - 1) & 1u));
           const u32* cs = coefs + (size_t)(cu * 2) * S;
           u32 g[S];
 #pragma unroll
@@ -411,6 +475,9 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
             u32 o[S];
             N::update(ld_num<L>(y, m, l, part), cr, ld_num<L>(x, m, l, part), ~0u, cim, ld_num<L>(x, m, l, part ^ 1),
                       (u32)-part, o);
+            if (glob && push_out)
+#pragma unroll
+              for (int q = 0; q < L / 2; ++q) push16(rpush + 16u * ((part * (L / 2) + q) * m + l), o + 4 * q, rbar);
             st_words<L>(y, m, l, part, o);
             if (glob) st_words<L>(pub, m, l, part, o);
           }
@@ -425,11 +492,12 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
           }
         }
         if (norm) MGS_TR(k, 5);
+        if (crit && sb == s0) ++pushes;  // column k + 1 was in this pass
         norm = false;
         sb += nb;
       } while (sb < wc);
       MGS_TR(k, 6);
-      if (!mine) {
+      if (!mine && !pushed) {
         __syncwarp();
         if (lane == 0 && alive) mbar_arrive(empty + st);
         if (++st == (u32)NS) {
@@ -442,7 +510,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     sync_warps();
     for (int s = tid; s <= wc; s += NW * 32) {
       const int k = s < wc ? col_of(s) - 1 : nc - 1;
-      if (k < 0 || (s == wc && jlast != nc - 1)) continue;
+      if (k < 0 || wc == 0 || (s == wc && jlast != nc - 1)) continue;
       u32 g[S], r[S];
 #pragma unroll
       for (int i = 0; i < S; ++i) {
@@ -478,6 +546,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
         ++own;
         continue;
       }
+      if (push_in && own < wc && k + 1 == col_of(own)) continue;  // pushed by the CTA before
       const u32 st = got % (u32)NS, turn = got / (u32)NS;
       if (turn > 0 && !mbar_wait(pr, empty + st, (turn - 1) & 1u)) break;
       if (!wait_word(pr.flags + k, kPublished)) break;
@@ -494,6 +563,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     }
   }
   MGS_TR(nc, 0);
+  if (pr.CL > 1) cooperative_groups::this_cluster().sync();  // no CTA leaves while a peer may still push to it
   grid_barrier(pr, epoch);
   MGS_TR(nc, 1);
 

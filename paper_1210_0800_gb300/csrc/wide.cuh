@@ -366,25 +366,16 @@ struct Wide {
   }
 
   // ---------------------------------------------------------------- division, square root
-  // floor(2^63 / (d + 1)) for a word d with its top bit set, or up to 2 below it
+  // 2^63 / (d + 1) for a word d with its top bit set, or up to 3 below it
   __host__ __device__ static __forceinline__ u32 reciprocal(u32 d) {
     const u64 d1 = (u64)d + 1;
 #if defined(__CUDA_ARCH__)
+    // below 2^63 / d1 by 2^-22 .. 2^-20 of it, then one Newton correction y + y (2^63 - d1 y) / 2^63
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rz(d)));
-    u64 x = (u64)__float2uint_rz(r * 0x1p62f) << 1;  // 2^63 / d to about 22 bits
-    long long err = (long long)((1ull << 63) - x * d1);
-    // one Newton correction x + x err / 2^63, then whole steps to an underestimate
-    x += (u64)(((err >> 18) * (long long)(x >> 3)) >> 42);
-    err = (long long)((1ull << 63) - x * d1);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (err < 0) {
-        --x;
-        err += (long long)d1;
-      }
-    if (err >= (long long)d1) ++x;
-    return x > 0xffffffffull ? 0xffffffffu : (u32)x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_ru(d)));
+    const u32 y = __float2uint_rz(r * (0x1p62f - 0x1p41f)) << 1;
+    const u64 e = (1ull << 63) - d1 * y;
+    return y + (u32)(((u64)y * (u32)(e >> 20)) >> 43);
 #else
     const u64 x = (1ull << 63) / d1;
     return x > 0xffffffffull ? 0xffffffffu : (u32)x;
