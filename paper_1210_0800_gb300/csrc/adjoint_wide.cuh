@@ -16,7 +16,7 @@ namespace mgs {
 
 // Shared memory: the sums of a solve; u, w, x (n elements), r, grad_b (m), as words; r_kk.
 __host__ __device__ inline size_t adjoint_wide_smem_bytes(int L, int max_m, int max_n) {
-  return (size_t)max_n * 2 * (L == 2 ? 24 : 48) + (3 * (size_t)max_n + 2 * (size_t)max_m) * 16 * L +
+  return (size_t)max_n * 2 * (L == 2 ? 32 : 48) + (3 * (size_t)max_n + 2 * (size_t)max_m) * 16 * L +
          (size_t)max_n * 8 * L + 64;
 }
 
@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
   using N = Wide<L>;
   using num = typename N::num;
   using sum = typename N::sum;
-  constexpr int SW = N::S, K = N::K, E = 2 * L, Q4 = L / 2, YW = L == 2 ? 6 : 12;
+  constexpr int SW = N::S, E = 2 * L, YW = kSumWords<L>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   extern __shared__ __align__(16) unsigned char asm_[];
   u32* ys = reinterpret_cast<u32*>(asm_);      // 2 n sums
@@ -37,27 +37,10 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
   u32* dw = gw + (size_t)ap.max_m * 2 * SW;    // r_kk
   int* sflag = reinterpret_cast<int*>(dw + (size_t)ap.max_n * SW);
   auto packed = [](int k, int j) { return (size_t)j * (j + 1) / 2 + k; };
-  auto ld_limbs = [&](const double* p, u32* o) {
+  auto ld_limbs_as_words = [&](const double* p, u32* o) {
     double v[L];
-    const double2* q = reinterpret_cast<const double2*>(p);
-#pragma unroll
-    for (int i = 0; i < Q4; ++i) {
-      const double2 d = q[i];
-      v[2 * i] = d.x;
-      v[2 * i + 1] = d.y;
-    }
+    ld_limbs<L>(p, v);
     N::of_limbs(v, o);
-  };
-  auto st_limbs = [&](double* p, const u32* o) {
-    double v[L];
-    N::to_limbs(o, v);
-    double2* q = reinterpret_cast<double2*>(p);
-#pragma unroll
-    for (int i = 0; i < Q4; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
-  };
-  auto cp = [&](u32* d, const u32* s) {
-#pragma unroll
-    for (int i = 0; i < SW; ++i) d[i] = s[i];
   };
 
   for (;;) {
@@ -85,26 +68,26 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
     u32* C = reinterpret_cast<u32*>(gA);  // c_kj at (k n + j) and (j n + k), k < j
     for (int i = tid; i < n; i += T) {
       u32 o[SW];
-      ld_limbs(R + packed(i, i) * E, o);
-      cp(dw + (size_t)i * SW, o);
+      ld_limbs_as_words(R + packed(i, i) * E, o);
+      sts_words<SW>(dw + (size_t)i * SW, o);
       if (!N::positive(o)) sflag[1] = ST_ERANK;
     }
     for (int i = tid; i < 2 * m; i += T) {
       u32 o[SW];
-      ld_limbs(rv + (size_t)i * L, o);
-      cp(rw + (size_t)i * SW, o);
+      ld_limbs_as_words(rv + (size_t)i * L, o);
+      sts_words<SW>(rw + (size_t)i * SW, o);
     }
     for (int i = tid; i < 2 * n; i += T) {
       u32 o[SW];
-      ld_limbs(xv + (size_t)i * L, o);
-      cp(xw + (size_t)i * SW, o);
-      ld_limbs(Gv + (size_t)i * L, o);
-      if (i < 2) cp(ww + (size_t)i * SW, o);  // (D u)_0
+      ld_limbs_as_words(xv + (size_t)i * L, o);
+      sts_words<SW>(xw + (size_t)i * SW, o);
+      ld_limbs_as_words(Gv + (size_t)i * L, o);
+      if (i < 2) sts_words<SW>(ww + (size_t)i * SW, o);  // (D u)_0
       const num v = N::unpack(o);
       sum a;
       N::clear(a);
       N::add(a, v.e + 4, v, 0u);
-      st_sum<L>(ys + (size_t)i * YW, a, v.e + 4);
+      st_item<L>(ys + (size_t)i * YW, a, v.e + 4);
     }
     __syncthreads();
     for (int idx = tid; idx < n * (n - 1); idx += T) {
@@ -114,10 +97,10 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
       while ((j + 1) * j / 2 <= pi) ++j;
       const int k = pi - j * (j - 1) / 2;
       u32 o[SW];
-      ld_limbs(R + packed(k, j) * E + p * L, o);
+      ld_limbs_as_words(R + packed(k, j) * E + p * L, o);
       N::div_words(o, dw + (size_t)k * SW, o);
-      cp(C + ((size_t)k * n + j) * 2 * SW + p * SW, o);
-      cp(C + ((size_t)j * n + k) * 2 * SW + p * SW, o);
+      sts_words<SW>(C + ((size_t)k * n + j) * 2 * SW + p * SW, o);
+      sts_words<SW>(C + ((size_t)j * n + k) * 2 * SW + p * SW, o);
     }
     __syncthreads();
     // Unit triangular solves: link k takes the unknown k off the rows on its far side (`up`: the
@@ -130,15 +113,14 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
           const int r = up ? k - 1 - (i >> 1) : k + 1 + (i >> 1), p = i & 1;
           u32 c1[SW], c2[SW];
           const u32* cc = C + ((size_t)k * n + r) * 2 * SW;
-          cp(c1, cc);
-          cp(c2, cc + SW);
+          lds_words<SW>(cc, c1);
+          lds_words<SW>(cc + SW, c2);
           u32* ya = ys + (size_t)(2 * r + p) * YW;
           const num cr = N::unpack(c1), ci = N::unpack(c2);
-          const num x1 = N::unpack(ww + (size_t)(2 * k + p) * SW), x2 = N::unpack(ww + (size_t)(2 * k + (p ^ 1)) * SW);
+          const num x1 = lds_num<L>(ww + (size_t)(2 * k + p) * SW), x2 = lds_num<L>(ww + (size_t)(2 * k + (p ^ 1)) * SW);
           sum a;
-#pragma unroll
-          for (int q = 0; q < K; ++q) a.a[q] = ya[q];
-          int Ex = (int)ya[K];
+          int Ex;
+          ld_item<L>(ya, a, Ex);
           const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
           if (need > Ex) {
             N::shift_sum(a, need - Ex);
@@ -149,7 +131,7 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
           if (i < 2)
             N::store(a, Ex, ww + (size_t)(2 * r + p) * SW);
           else
-            st_sum<L>(ya, a, Ex);
+            st_item<L>(ya, a, Ex);
         }
         __syncthreads();
       }
@@ -160,14 +142,14 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
       u32 o[SW], d[SW];
       const u32* dk = dw + (size_t)(i >> 1) * SW;
       N::div_words(ww + (size_t)i * SW, dk, o);
-      cp(uw + (size_t)i * SW, o);
+      sts_words<SW>(uw + (size_t)i * SW, o);
       N::div_words(o, dk, d);
-      if ((i >> 1) == n - 1) cp(ww + (size_t)i * SW, d);
+      if ((i >> 1) == n - 1) sts_words<SW>(ww + (size_t)i * SW, d);
       const num v = N::unpack(d);
       sum a;
       N::clear(a);
       N::add(a, v.e + 4, v, 0u);
-      st_sum<L>(ys + (size_t)i * YW, a, v.e + 4);
+      st_item<L>(ys + (size_t)i * YW, a, v.e + 4);
     }
     __syncthreads();
     solve(true);
@@ -183,12 +165,12 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
         u32 o[SW], t[SW];
 #pragma unroll
         for (int q = 0; q < SW; ++q) o[q] = 0u;
-        if (k < n) ld_limbs(Q + ((size_t)k * m + i) * E + p * L, o);
+        if (k < n) ld_limbs_as_words(Q + ((size_t)k * m + i) * E + p * L, o);
 #pragma unroll
         for (int q = 0; q < SW; ++q) t[q] = __shfl_xor_sync(0xffffffffu, o[q], 16);
         const u32* uk = uw + (size_t)min(k, n - 1) * 2 * SW;
         // re: qr ur - qi ui, im: qi ur + qr ui (a zero Q past the last column adds nothing)
-        const num q1 = N::unpack(o), q2 = N::unpack(t), ur = N::unpack(uk), ui = N::unpack(uk + SW);
+        const num q1 = N::unpack(o), q2 = N::unpack(t), ur = lds_num<L>(uk), ui = lds_num<L>(uk + SW);
         const int need = max(q1.e + ur.e, q2.e + ui.e) + N::SUMBITS;
         if (need > Ex) {
           N::shift_sum(a, need - Ex);
@@ -202,8 +184,8 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
       u32 o[SW];
       N::store(a, top, o);
       if ((lane & 15) == 0) {
-        cp(gw + (size_t)(2 * i + p) * SW, o);
-        st_limbs(gb + (size_t)(2 * i + p) * L, o);
+        sts_words<SW>(gw + (size_t)(2 * i + p) * SW, o);
+        st_limbs<L>(gb + (size_t)(2 * i + p) * L, o);
       }
     }
     __syncthreads();
@@ -211,10 +193,10 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
     for (int t = tid; t < 2 * m * n; t += T) {
       const int p = t & 1, rest = t >> 1;
       const int j = rest / m, i = rest - j * m;
-      const num wr = N::unpack(ww + (size_t)2 * j * SW), wi = N::unpack(ww + (size_t)(2 * j + 1) * SW);
-      const num xr = N::unpack(xw + (size_t)2 * j * SW), xi = N::unpack(xw + (size_t)(2 * j + 1) * SW);
-      const num r1 = N::unpack(rw + (size_t)(2 * i + p) * SW), r2 = N::unpack(rw + (size_t)(2 * i + (p ^ 1)) * SW);
-      const num g1 = N::unpack(gw + (size_t)(2 * i + p) * SW), g2 = N::unpack(gw + (size_t)(2 * i + (p ^ 1)) * SW);
+      const num wr = lds_num<L>(ww + (size_t)2 * j * SW), wi = lds_num<L>(ww + (size_t)(2 * j + 1) * SW);
+      const num xr = lds_num<L>(xw + (size_t)2 * j * SW), xi = lds_num<L>(xw + (size_t)(2 * j + 1) * SW);
+      const num r1 = lds_num<L>(rw + (size_t)(2 * i + p) * SW), r2 = lds_num<L>(rw + (size_t)(2 * i + (p ^ 1)) * SW);
+      const num g1 = lds_num<L>(gw + (size_t)(2 * i + p) * SW), g2 = lds_num<L>(gw + (size_t)(2 * i + (p ^ 1)) * SW);
       // re: wr rr + wi ri - xr gr - xi gi, im: wr ri - wi rr - xr gi + xi gr
       const int Ex = max(max(wr.e + r1.e, wi.e + r2.e), max(xr.e + g1.e, xi.e + g2.e)) + 3;
       sum a;
@@ -223,7 +205,7 @@ __global__ void __launch_bounds__(T) mgs_adjoint_wide_kernel(AdjParams ap) {
       N::mac2(a, Ex, xr, g1, ~0u, xi, g2, p ? 0u : ~0u);
       u32 o[SW];
       N::store(a, Ex, o);
-      st_limbs(gA + (size_t)t * L, o);
+      st_limbs<L>(gA + (size_t)t * L, o);
     }
     __syncthreads();
     if (tid == 0) ap.status[sys] = sflag[1];

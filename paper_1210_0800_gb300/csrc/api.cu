@@ -173,20 +173,26 @@ bool compute_plan(int L, int m, int n, int aug, int want, int h0, int T0, int cp
   return true;
 }
 
-// The column kernel's layout (double-double and quad-double, default choices only): whole
+// The column kernel's layout (default choices only): whole
 // columns per CTA.  Replaces the plan made before it when a CTA's columns and two pivot
 // stages fit in shared memory; the workspace stays at least what that plan asked for.
 void column_plan(Plan& pl) {
   const int L = pl.L, m = pl.m, nc = pl.nc;
-  if (L == 1 || m > 2048) return;
+  if (m > 2048) return;
   const int sms = device_sms();
-  int bw = 1, warps = mgs::kColWarps, stages = 4, first = 1;
+  const int bw = 1, first = 1;
+  int stages = 4;
   const int halves = (m + 15) / 16;  // 16-row pieces of a column
+  // warps on columns: 15, or 12 where the pieces take no more rounds (two thirds of the warps in
+  // the dot products, all in the updates); us at 12 / 15: 256 rows DD 1370 / 1411, 128 DD 539 / 547,
+  // 128 QD 723 / 737, but 200 QD 1423 / 1355
+  auto rounds = [&](int nw) { return (halves + nw * 2 / 3 - 1) / (nw * 2 / 3) + (halves + nw - 1) / nw; };
+  int warps = rounds(12) <= rounds(mgs::kColWarps) ? 12 : mgs::kColWarps;
   // clusters of 8 CTAs (7 of 8 pivots are pushed to their next owner) when they leave a CTA no
-  // more columns than CTAs on all SMs would own; else of 4 or 2, or none
-  // (measured, us with / without: n = 32 DD 128 / 145, 256 1413 / 1531, 320x256 QD 2253 / 2347; with
-  // more than two columns a CTA the other columns' work hides the hand-off and the SMs that
-  // clusters leave idle cost more: 512 QD 7710 / 7561)
+  // more columns than CTAs on all SMs would own; else of 4 or 2, or none.  Measured, us with /
+  // without: n = 32 DD 128 / 145, 256 DD 1413 / 1531, 320x256 QD 2253 / 2347; with more than two
+  // columns a CTA the other columns' work hides the hand-off and the SMs that clusters leave
+  // idle cost more: 512 QD 7710 / 7561.
   const int w = (nc + sms - 1) / sms * bw;
   int CL = w <= 2 ? 8 : 1;
   if (warps > halves * (w + 1)) warps = halves * (w + 1);  // a pass: w columns and the norm

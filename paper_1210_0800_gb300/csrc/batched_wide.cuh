@@ -25,7 +25,7 @@ namespace mgs {
 
 // Bytes of the back substitution's sums and unknowns.
 __host__ __device__ inline size_t batched_backsub_bytes(int L, int max_n) {
-  return (size_t)max_n * (2 * (L == 2 ? 24 : 48) + 16 * L);
+  return (size_t)max_n * (2 * (L == 2 ? 32 : 48) + 16 * L);
 }
 // The largest back substitution kept in shared memory: two CTAs still fit an SM.  Larger ones
 // keep their sums in the global scratch.
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
   using num = typename N::num;
   using sum = typename N::sum;
   constexpr int SW = N::S, K = N::K, E = 2 * L, Q4 = L / 2, NW = T / 32;
-  constexpr int PW = L == 2 ? 6 : 10, YW = L == 2 ? 6 : 12;
+  constexpr int PW = L == 2 ? 6 : 10, YW = kSumWords<L>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int part = lane >> 4, lr = lane & 15;
   const int rank = (int)(blockIdx.x % S);
@@ -90,28 +90,10 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
       o[4 * i + 3] = v.w;
     }
   };
-  auto ld_part_cg = [&](const u32* p, u32* o) {
-    const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-    for (int i = 0; i < Q4; ++i) {
-      const uint4 v = __ldcg(q + i);
-      o[4 * i] = v.x;
-      o[4 * i + 1] = v.y;
-      o[4 * i + 2] = v.z;
-      o[4 * i + 3] = v.w;
-    }
-  };
   auto st_part = [&](u32* p, const u32* o) {
     uint4* q = reinterpret_cast<uint4*>(p);
 #pragma unroll
     for (int i = 0; i < Q4; ++i) q[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-  };
-  auto st_limbs = [&](double* p, const u32* o) {
-    double v[L];
-    N::to_limbs(o, v);
-    double2* q = reinterpret_cast<double2*>(p);
-#pragma unroll
-    for (int i = 0; i < Q4; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
   };
 
   for (;;) {
@@ -174,7 +156,7 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
         N::clear(a);
         for (int i = tid; i < m * 2; i += T) {
           u32 v[SW];
-          ld_part_cg(ck + (size_t)i * SW, v);
+          ld_part_cg<L>(ck + (size_t)i * SW, v);
           st_words<L>(piv, m, i >> 1, i & 1, v);
           const num x = N::unpack(v);
           const int need = 2 * x.e + N::SUMBITS;
@@ -290,7 +272,7 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
     // q_j = a_j / r_jj of the own columns; the last column (b) is the residual
     for (int j = rank; j < nc; j += S) {
       u32 r[SW];
-      ld_part_cg(Rd + (size_t)j * SW, r);
+      ld_part_cg<L>(Rd + (size_t)j * SW, r);
       const bool q = j < n;
       if (q && !N::positive(r)) continue;
       double* cj = col(j);
@@ -298,7 +280,7 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
         u32 v[SW];
         ld_part(reinterpret_cast<u32*>(cj + (size_t)i * L), v);
         if (q) N::div_words(v, r, v);
-        st_limbs(cj + (size_t)i * L, v);
+        st_limbs<L>(cj + (size_t)i * L, v);
       }
     }
     // the rest is rank 0's: R, back substitution, x, status
@@ -313,13 +295,13 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
         const int k = pi - j * (j + 1) / 2;
         double* dst = Ro + packed(k, j) * E + p * L;
         u32 r[SW], v[SW];
-        ld_part_cg(Rd + (size_t)k * SW, r);
+        ld_part_cg<L>(Rd + (size_t)k * SW, r);
         if (k < j) {
-          ld_part_cg(Rp + packed(k, j) * 2 * SW + p * SW, v);
+          ld_part_cg<L>(Rp + packed(k, j) * 2 * SW + p * SW, v);
           N::mul_words(v, r, v);
-          st_limbs(dst, v);
+          st_limbs<L>(dst, v);
         } else if (p == 0) {
-          st_limbs(dst, r);
+          st_limbs<L>(dst, r);
         } else {
 #pragma unroll
           for (int q = 0; q < L; ++q) dst[q] = 0.0;
@@ -333,7 +315,7 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
     __syncthreads();
     for (int i = tid; i < n * 2; i += T) {
       u32 v[SW];
-      ld_part_cg(Yv + (size_t)i * SW, v);
+      ld_part_cg<L>(Yv + (size_t)i * SW, v);
       if ((i >> 1) == n - 1) {
 #pragma unroll
         for (int q = 0; q < SW; ++q) xs[(size_t)i * SW + q] = v[q];
@@ -342,15 +324,15 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
       sum a;
       N::clear(a);
       N::add(a, v0.e + 4, v0, 0u);
-      st_sum<L>(ys + (size_t)i * YW, a, v0.e + 4);
+      st_item<L>(ys + (size_t)i * YW, a, v0.e + 4);
     }
     u32 nr[SW], ni[SW];  // the next link's coefficients of this thread's first item
     auto fetch = [&](int k) {
       const int it = 2 * k - 1 - tid;
       if (it >= 0) {
         const u32* c2 = Rp + packed(it >> 1, k) * 2 * SW;
-        ld_part_cg(c2, nr);
-        ld_part_cg(c2 + SW, ni);
+        ld_part_cg<L>(c2, nr);
+        ld_part_cg<L>(c2 + SW, ni);
       }
     };
     if (n > 1) fetch(n - 1);
@@ -368,11 +350,10 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
         const int p = it & 1;
         u32* ya = ys + (size_t)it * YW;
         const num cr = N::unpack(c1), ci = N::unpack(c2);
-        const num x1 = N::unpack(xs + (size_t)(2 * k + p) * SW), x2 = N::unpack(xs + (size_t)(2 * k + (p ^ 1)) * SW);
+        const num x1 = lds_num<L>(xs + (size_t)(2 * k + p) * SW), x2 = lds_num<L>(xs + (size_t)(2 * k + (p ^ 1)) * SW);
         sum a;
-#pragma unroll
-        for (int q = 0; q < K; ++q) a.a[q] = ya[q];
-        int Ex = (int)ya[K];
+        int Ex;
+        ld_item<L>(ya, a, Ex);
         // two products of less than 2^(need - 13) in each of at most 2^11 links: |a| < 2^(Ex - 1)
         const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
         if (need > Ex) {
@@ -383,16 +364,16 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
         if ((it >> 1) == k - 1)
           N::store(a, Ex, xs + (size_t)it * SW);
         else
-          st_sum<L>(ya, a, Ex);
+          st_item<L>(ya, a, Ex);
         if (it >= T) {
           const u32* cn = Rp + packed((it - T) >> 1, k) * 2 * SW;
-          ld_part_cg(cn, c1);
-          ld_part_cg(cn + SW, c2);
+          ld_part_cg<L>(cn, c1);
+          ld_part_cg<L>(cn + SW, c2);
         }
       }
       __syncthreads();
     }
-    for (int i = tid; i < n * 2; i += T) st_limbs(xv + (size_t)i * L, xs + (size_t)i * SW);
+    for (int i = tid; i < n * 2; i += T) st_limbs<L>(xv + (size_t)i * L, xs + (size_t)i * SW);
     __syncthreads();
     if (tid == 0) {
       // the input check comes first: a non-finite entry in any column wins over the rank

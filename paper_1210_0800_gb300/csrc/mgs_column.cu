@@ -5,7 +5,9 @@
 namespace mgs {
 namespace {
 const void* column_kernel(int L) {
-  return L == 2 ? (const void*)mgs_column_kernel<2> : (const void*)mgs_column_kernel<4>;
+  return L == 1   ? (const void*)mgs_column_kernel<1>
+         : L == 2 ? (const void*)mgs_column_kernel<2>
+                  : (const void*)mgs_column_kernel<4>;
 }
 }  // namespace
 

@@ -1,6 +1,6 @@
 // Single-system MGS least squares with whole columns per CTA and no grid-wide barrier during
 // the sweep (Section 3, Figure 1 and Eq. 1; Section 6), on the wide binary arithmetic of
-// wide.cuh.
+// wide.cuh (complex double: FP64, wide_d.cuh).
 //
 // What bounds it: the chain of n dependent steps.  Pivot k must reach the owner of column
 // k+1, which projects, divides, updates and passes pivot k+1 on; the other columns of a step
@@ -40,6 +40,7 @@
 
 #include "mgs_kernel.cuh"
 #include "wide.cuh"
+#include "wide_d.cuh"
 
 namespace mgs {
 
@@ -71,7 +72,7 @@ constexpr int kColThreads = 32 * (kColWarps + 1);  // and the receiving one
 
 constexpr unsigned kPublished = 16;                // > kColWarps: shares of the warps that publish add up to it
 
-__host__ __device__ inline size_t col_part_words(int L) { return L == 2 ? 6 : 10; }  // a sum and its exponent
+__host__ __device__ inline size_t col_part_words(int L) { return L == 1 ? 4 : L == 2 ? 6 : 10; }  // a sum and its exponent
 // shared memory after the stages and the tile: partial sums (two parts a warp), coefficients,
 // G_kk of the pivots before the own columns and of the last one, G_kk of this step, mbarriers
 __host__ __device__ inline size_t col_smem_bytes(int L, int m, int w, int stages, int CL) {
@@ -84,7 +85,7 @@ __host__ __device__ inline size_t col_smem_bytes(int L, int m, int w, int stages
 // back substitution: the sums, x, and a ring of columns of coefficients
 constexpr int kColBS = 4;
 __host__ __device__ inline size_t col_backsub_bytes(int L, int n) {
-  return (size_t)n * 2 * (L == 2 ? 24 : 48) + (size_t)n * 16 * L + (size_t)kColBS * n * 16 * L + 8 * kColBS + 64;
+  return (size_t)n * 2 * (L == 1 ? 16 : L == 2 ? 32 : 48) + (size_t)n * 16 * L + (size_t)kColBS * n * 16 * L + 8 * kColBS + 64;
 }
 
 // ------------------------------------------------------------------ PTX
@@ -131,6 +132,11 @@ __device__ __forceinline__ void push16(u32 dst, const u32* w, u32 bar) {
                "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(bar)
                : "memory");
 }
+__device__ __forceinline__ void push8(u32 dst, const u32* w, u32 bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(dst),
+               "r"(w[0]), "r"(w[1]), "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, u32 bytes, u64* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_addr(dst)),
@@ -159,30 +165,109 @@ __device__ __forceinline__ bool mbar_wait(const ColParams& pr, u64* bar, u32 par
 }
 
 // ------------------------------------------------------------------ planes
-// A column in shared or published memory: uint4 plane q of row l at q * m + l; part p of an
-// element is planes p * L / 2 .. (L words of 16 bytes per element).
+// A column in shared or published memory.  L > 1: uint4 plane q of row l at q * m + l, part p of
+// an element in planes p L / 2 .. (L uint4 per element); L = 1: an element's two doubles in
+// uint4 l.
+template <int L>
+__device__ __forceinline__ void ld_words(const uint4* col, int m, int l, int part, u32* w) {
+  if constexpr (L == 1) {
+    const uint2 v = reinterpret_cast<const uint2*>(col)[2 * (size_t)l + part];
+    w[0] = v.x;
+    w[1] = v.y;
+  } else {
+#pragma unroll
+    for (int q = 0; q < L / 2; ++q) {
+      const uint4 v = col[(size_t)(part * (L / 2) + q) * m + l];
+      w[4 * q] = v.x;
+      w[4 * q + 1] = v.y;
+      w[4 * q + 2] = v.z;
+      w[4 * q + 3] = v.w;
+    }
+  }
+}
 template <int L>
 __device__ __forceinline__ typename Wide<L>::num ld_num(const uint4* col, int m, int l, int part) {
   u32 w[2 * L];
-#pragma unroll
-  for (int q = 0; q < L / 2; ++q) {
-    const uint4 v = col[(size_t)(part * (L / 2) + q) * m + l];
-    w[4 * q] = v.x;
-    w[4 * q + 1] = v.y;
-    w[4 * q + 2] = v.z;
-    w[4 * q + 3] = v.w;
-  }
+  ld_words<L>(col, m, l, part, w);
   return Wide<L>::unpack(w);
 }
 template <int L>
 __device__ __forceinline__ void st_words(uint4* col, int m, int l, int part, const u32* w) {
+  if constexpr (L == 1) {
+    reinterpret_cast<uint2*>(col)[2 * (size_t)l + part] = make_uint2(w[0], w[1]);
+  } else {
 #pragma unroll
-  for (int q = 0; q < L / 2; ++q)
-    col[(size_t)(part * (L / 2) + q) * m + l] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    for (int q = 0; q < L / 2; ++q)
+      col[(size_t)(part * (L / 2) + q) * m + l] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+  }
+}
+// the same into a peer's memory (dst: its column)
+template <int L>
+__device__ __forceinline__ void push_words(u32 dst, int m, int l, int part, const u32* w, u32 bar) {
+  if constexpr (L == 1) {
+    push8(dst + 8u * (2 * l + part), w, bar);
+  } else {
+#pragma unroll
+    for (int q = 0; q < L / 2; ++q) push16(dst + 16u * ((part * (L / 2) + q) * m + l), w + 4 * q, bar);
+  }
+}
+// one part of an element in row-major global scratch (past L1), and a part's limbs
+template <int L>
+__device__ __forceinline__ void ld_part_cg(const u32* p, u32* o) {
+  if constexpr (L == 1) {
+    const uint2 v = __ldcg(reinterpret_cast<const uint2*>(p));
+    o[0] = v.x;
+    o[1] = v.y;
+  } else {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+#pragma unroll
+    for (int i = 0; i < L / 2; ++i) {
+      const uint4 v = __ldcg(q + i);
+      o[4 * i] = v.x;
+      o[4 * i + 1] = v.y;
+      o[4 * i + 2] = v.z;
+      o[4 * i + 3] = v.w;
+    }
+  }
+}
+template <int L>
+__device__ __forceinline__ void st_part_cg(u32* p, const u32* o) {
+  if constexpr (L == 1) {
+    __stcg(reinterpret_cast<uint2*>(p), make_uint2(o[0], o[1]));
+  } else {
+#pragma unroll
+    for (int i = 0; i < L / 2; ++i)
+      __stcg(reinterpret_cast<uint4*>(p) + i, make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]));
+  }
+}
+template <int L>
+__device__ __forceinline__ void ld_limbs(const double* p, double* v) {
+  if constexpr (L == 1) {
+    v[0] = p[0];
+  } else {
+#pragma unroll
+    for (int i = 0; i < L / 2; ++i) {
+      const double2 d = reinterpret_cast<const double2*>(p)[i];
+      v[2 * i] = d.x;
+      v[2 * i + 1] = d.y;
+    }
+  }
+}
+template <int L>
+__device__ __forceinline__ void st_limbs(double* p, const u32* o) {
+  double v[L];
+  Wide<L>::to_limbs(o, v);
+  if constexpr (L == 1) {
+    p[0] = v[0];
+  } else {
+#pragma unroll
+    for (int i = 0; i < L / 2; ++i) reinterpret_cast<double2*>(p)[i] = make_double2(v[2 * i], v[2 * i + 1]);
+  }
 }
 // the larger biased exponent of an element's parts
 template <int L>
 __device__ __forceinline__ int ld_exp(const uint4* col, int m, int l) {
+  if (L == 1) return 0;
   const u32* c = reinterpret_cast<const u32*>(col);
   if (L == 2) {
     const u32 a = c[4 * (size_t)l] & 0xffffu, b = c[4 * ((size_t)m + l)] & 0xffffu;
@@ -200,10 +285,63 @@ __device__ __forceinline__ void lane_sum(typename Wide<L>::sum& s) {
     u32 t[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) t[q] = __shfl_xor_sync(0xffffffffu, s.a[q], off);
-    add_words<K>(s.a, t);
+    Wide<L>::add_sum(s, t);
   }
 }
-// a sum and its exponent in shared memory, and back
+// N aligned words by vector loads and stores: scalar ones, at strides of several
+// words from lane to lane, conflict on the banks.
+template <int N>
+__device__ __forceinline__ void lds_words(const u32* p, u32* o) {
+  if constexpr (N == 2) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p);
+    o[0] = v.x;
+    o[1] = v.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) {
+      const uint4 v = reinterpret_cast<const uint4*>(p)[i];
+      o[4 * i] = v.x;
+      o[4 * i + 1] = v.y;
+      o[4 * i + 2] = v.z;
+      o[4 * i + 3] = v.w;
+    }
+  }
+}
+template <int N>
+__device__ __forceinline__ void sts_words(u32* p, const u32* o) {
+  if constexpr (N == 2) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(o[0], o[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i)
+      reinterpret_cast<uint4*>(p)[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+  }
+}
+// The sums of a back substitution: words of each with its exponent, padded.
+template <int L>
+constexpr int kSumWords = L == 1 ? 4 : L == 2 ? 8 : 12;
+template <int L>
+__device__ __forceinline__ void ld_item(const u32* p, typename Wide<L>::sum& s, int& E) {
+  u32 w[kSumWords<L>];
+  lds_words<kSumWords<L>>(p, w);
+#pragma unroll
+  for (int q = 0; q < Wide<L>::K; ++q) s.a[q] = w[q];
+  E = (int)w[Wide<L>::K];
+}
+template <int L>
+__device__ __forceinline__ void st_item(u32* p, const typename Wide<L>::sum& s, int E) {
+  u32 w[kSumWords<L>];
+#pragma unroll
+  for (int q = 0; q < kSumWords<L>; ++q) w[q] = q < Wide<L>::K ? s.a[q] : (u32)E;
+  sts_words<kSumWords<L>>(p, w);
+}
+template <int L>
+__device__ __forceinline__ typename Wide<L>::num lds_num(const u32* p) {
+  u32 w[2 * L];
+  lds_words<2 * L>(p, w);
+  return Wide<L>::unpack(w);
+}
+// a sum and its exponent in shared memory
 template <int L>
 __device__ __forceinline__ void st_sum(u32* p, const typename Wide<L>::sum& s, int E) {
 #pragma unroll
@@ -227,7 +365,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   uint4* stage = reinterpret_cast<uint4*>(csm);
   uint4* push = stage + (size_t)NS * colv;  // the pivot before an own column, from the CTA before
   uint4* tile = push + (pr.CL > 1 ? colv : 0);
-  constexpr int PW = L == 2 ? 6 : 10;
+  constexpr int PW = L == 1 ? 4 : L == 2 ? 6 : 10;
   u32* parts = reinterpret_cast<u32*>(tile + (size_t)w * colv);  // a warp's sums: 2 x PW
   u32* coefs = parts + (size_t)kColWarps * 2 * PW;               // c_kj of the pass's columns: 2 S words each
   u32* gown = coefs + (size_t)kColWarps * 2 * S;                 // G_kk of the pivot before own column s; [w]: the last
@@ -259,14 +397,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     for (int idx = tid; idx < wc * m * 2; idx += nthreads) {
       const int part = idx & 1, rest = idx >> 1;
       const int s = rest / m, l = rest % m;
-      const double2* src = reinterpret_cast<const double2*>(gcol(col_of(s)) + (size_t)l * E + part * L);
       double v[L];
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        const double2 d = src[q];
-        v[2 * q] = d.x;
-        v[2 * q + 1] = d.y;
-      }
+      ld_limbs<L>(gcol(col_of(s)) + (size_t)l * E + part * L, v);
 #pragma unroll
       for (int q = 0; q < L; ++q) bad |= !finite64(v[q]);
       u32 o[S];
@@ -414,7 +546,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
               u32 t[K], g[S];
 #pragma unroll
               for (int q = 0; q < K; ++q) t[q] = __shfl_xor_sync(0xffffffffu, a.a[q], 16);
-              add_words<K>(a.a, t);
+              N::add_sum(a, t);
               N::store(a, Ex, g);
               if (lane == 0) {
 #pragma unroll
@@ -435,22 +567,18 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
         if (head) {
           const int j = col_of(sb + cd);
           u32 g[S], q[S], f;
-#pragma unroll
-          for (int i = 0; i < S; ++i) g[i] = gcur[i];
+          lds_words<S>(gcur, g);
           v = N::quotient(v, N::unpack(g), f);
           N::pack(v, f, q);
           if (lr == 0) {
             const bool ok = N::positive(g);
             u32* cs = coefs + (size_t)(cd * 2 + part) * S;
-            uint4* dst = reinterpret_cast<uint4*>(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S);
 #pragma unroll
             for (int i = 0; i < S; ++i) {
               q[i] = ok ? q[i] : 0u;
               cs[i] = q[i];
             }
-#pragma unroll
-            for (int i = 0; i < S / 4; ++i)
-              __stcg(dst + i, make_uint4(q[4 * i], q[4 * i + 1], q[4 * i + 2], q[4 * i + 3]));
+            st_part_cg<L>(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S, q);
           }
         }
         if (norm) MGS_TR(k, 4);
@@ -464,20 +592,12 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
           if (glob && push_out && pushes > 0 && alive)
             alive = __all_sync(0xffffffffu, mbar_wait<true>(pr, pempty, (u32)(pushes - 1) & 1u));
           const u32* cs = coefs + (size_t)(cu * 2) * S;
-          u32 g[S];
-#pragma unroll
-          for (int i = 0; i < S; ++i) g[i] = cs[i];
-          const num cr = N::unpack(g);
-#pragma unroll
-          for (int i = 0; i < S; ++i) g[i] = cs[S + i];
-          const num cim = N::unpack(g);
+          const num cr = lds_num<L>(cs), cim = lds_num<L>(cs + S);
           for (int l = su * 16 + lr; l < m; l += wpu * 16) {  // re: y - cr xr + ci xi, im: y - cr xi - ci xr
             u32 o[S];
             N::update(ld_num<L>(y, m, l, part), cr, ld_num<L>(x, m, l, part), ~0u, cim, ld_num<L>(x, m, l, part ^ 1),
                       (u32)-part, o);
-            if (glob && push_out)
-#pragma unroll
-              for (int q = 0; q < L / 2; ++q) push16(rpush + 16u * ((part * (L / 2) + q) * m + l), o + 4 * q, rbar);
+            if (glob && push_out) push_words<L>(rpush, m, l, part, o, rbar);
             st_words<L>(y, m, l, part, o);
             if (glob) st_words<L>(pub, m, l, part, o);
           }
@@ -574,24 +694,6 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     else if (ld_acquire_u32(&pr.sync[3]))
       set_status(pr.status, ST_ERANK);
   }
-  auto ld_w = [&](const u32* p, u32* o) {
-    const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-    for (int i = 0; i < S / 4; ++i) {
-      const uint4 v = __ldcg(q + i);
-      o[4 * i] = v.x;
-      o[4 * i + 1] = v.y;
-      o[4 * i + 2] = v.z;
-      o[4 * i + 3] = v.w;
-    }
-  };
-  auto st_limbs = [&](double* p, const u32* o) {
-    double v[L];
-    N::to_limbs(o, v);
-    double2* q = reinterpret_cast<double2*>(p);
-#pragma unroll
-    for (int i = 0; i < L / 2; ++i) q[i] = make_double2(v[2 * i], v[2 * i + 1]);
-  };
   // Q, the residual, R, z of the own columns
   auto outputs = [&](int first, int count) {  // by `count` threads from thread `first` on
     const int t0 = tid - first;
@@ -599,21 +701,13 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       const int part = idx & 1, rest = idx >> 1;
       const int s = rest / m, l = rest % m, j = col_of(s);
       u32 a[S], r[S], o[S];
-      const uint4* col = tile + (size_t)s * colv;
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        const uint4 v = col[(size_t)(part * (L / 2) + q) * m + l];
-        a[4 * q] = v.x;
-        a[4 * q + 1] = v.y;
-        a[4 * q + 2] = v.z;
-        a[4 * q + 3] = v.w;
-      }
+      ld_words<L>(tile + (size_t)s * colv, m, l, part, a);
       double* dst = gcol(j) + (size_t)l * E + part * L;
       if (j < pr.n) {
-        ld_w(pr.Rd + (size_t)j * S, r);
+        ld_part_cg<L>(pr.Rd + (size_t)j * S, r);
         if (!N::positive(r)) continue;
         N::div_words(a, r, o);
-        st_limbs(dst, o);
+        st_limbs<L>(dst, o);
       } else {
         // the residual; an entry that no projection changed is left as the caller wrote it
         double v[L];
@@ -623,7 +717,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
         bool same = true;
 #pragma unroll
         for (int q = 0; q < S; ++q) same &= o[q] == a[q];
-        if (!same) st_limbs(dst, a);
+        if (!same) st_limbs<L>(dst, a);
       }
     }
     if (pr.R)
@@ -633,14 +727,14 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
         for (int idx = t0; idx < 2 * j + 2; idx += count) {
           const int k = idx >> 1, part = idx & 1;
           u32 a[S], r[S], o[S];
-          ld_w(pr.Rd + (size_t)k * S, r);
+          ld_part_cg<L>(pr.Rd + (size_t)k * S, r);
           double* dst = pr.R + ((size_t)j * pr.ldr + k) * E + part * L;
           if (k < j) {
-            ld_w(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S, a);
+            ld_part_cg<L>(pr.C + ((size_t)j * (j - 1) / 2 + k) * 2 * S + part * S, a);
             N::mul_words(a, r, o);
-            st_limbs(dst, o);
+            st_limbs<L>(dst, o);
           } else if (part == 0) {
-            st_limbs(dst, r);
+            st_limbs<L>(dst, r);
           } else {
 #pragma unroll
             for (int q = 0; q < L; ++q) dst[q] = 0.0;
@@ -649,8 +743,8 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       }
     if (pr.aug && pr.z && jlast == nc - 1 && t0 == 0) {
       u32 r[S];
-      ld_w(pr.Rd + (size_t)(nc - 1) * S, r);
-      st_limbs(pr.z, r);
+      ld_part_cg<L>(pr.Rd + (size_t)(nc - 1) * S, r);
+      st_limbs<L>(pr.z, r);
     }
   };
   outputs(0, nthreads);
@@ -660,7 +754,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   // ---------------------------------------------------------------- back substitution (CTA 0)
   // x_k = c_kn - sum_{j > k} c_kj x_j.  Item i = 2 row + part.
   const int n = pr.n;
-  constexpr int SW = L == 2 ? 6 : 12;                            // a sum and its exponent, padded
+  constexpr int SW = kSumWords<L>;
   u32* ys = reinterpret_cast<u32*>(csm);                         // 2 n sums; the tile is no longer needed
   u32* y = ys + (size_t)2 * n * SW;                              // x, stored form
   uint4* ring = reinterpret_cast<uint4*>(y + (size_t)2 * n * S);  // column k of the coefficients in slot k % 4
@@ -682,7 +776,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     for (int i = 0; i < kColBS && n - 1 - i > 0; ++i) fetch(n - 1 - i, i);
   for (int i = tid; i < n * 2; i += nthreads) {
     u32 v[S];
-    ld_w(pr.C + ((size_t)n * (n - 1) / 2) * 2 * S + (size_t)i * S, v);
+    ld_part_cg<L>(pr.C + ((size_t)n * (n - 1) / 2) * 2 * S + (size_t)i * S, v);
     if ((i >> 1) == n - 1) {
 #pragma unroll
       for (int q = 0; q < S; ++q) y[(size_t)i * S + q] = v[q];
@@ -691,7 +785,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     sum a;
     N::clear(a);
     N::add(a, v0.e + 4, v0, 0u);
-    st_sum<L>(ys + (size_t)i * SW, a, v0.e + 4);
+    st_item<L>(ys + (size_t)i * SW, a, v0.e + 4);
   }
   __syncthreads();
   bool live = true;
@@ -703,12 +797,11 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       const int p = it & 1;
       u32* ya = ys + (size_t)it * SW;
       const u32* c2 = col + (size_t)(it >> 1) * 2 * S;
-      const num cr = N::unpack(c2), ci = N::unpack(c2 + S);
-      const num x1 = N::unpack(y + (size_t)(2 * k + p) * S), x2 = N::unpack(y + (size_t)(2 * k + (p ^ 1)) * S);
+      const num cr = lds_num<L>(c2), ci = lds_num<L>(c2 + S);
+      const num x1 = lds_num<L>(y + (size_t)(2 * k + p) * S), x2 = lds_num<L>(y + (size_t)(2 * k + (p ^ 1)) * S);
       sum a;
-#pragma unroll
-      for (int q = 0; q < K; ++q) a.a[q] = ya[q];
-      int Ex = (int)ya[K];
+      int Ex;
+      ld_item<L>(ya, a, Ex);
       // two products of less than 2^(need - 13) in each of at most 2^11 links: |a| < 2^(Ex - 1)
       const int need = max(cr.e + x1.e, ci.e + x2.e) + N::SUMBITS;
       if (need > Ex) {
@@ -717,9 +810,11 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       }
       N::mac2(a, Ex, cr, x1, ~0u, ci, x2, (u32)-p);
       if ((it >> 1) == k - 1) {
-        N::store(a, Ex, y + (size_t)it * S);
+        u32 o[S];
+        N::store(a, Ex, o);
+        sts_words<S>(y + (size_t)it * S, o);
       } else {
-        st_sum<L>(ya, a, Ex);
+        st_item<L>(ya, a, Ex);
       }
     }
     __syncthreads();
@@ -728,7 +823,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       fetch(k - kColBS, i + kColBS);
     }
   }
-  for (int i = tid; i < n * 2; i += nthreads) st_limbs(pr.x + (size_t)i * L, y + (size_t)i * S);
+  for (int i = tid; i < n * 2; i += nthreads) st_limbs<L>(pr.x + (size_t)i * L, y + (size_t)i * S);
   MGS_TR(nc, 3);
 }
 

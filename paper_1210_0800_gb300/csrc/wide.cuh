@@ -261,6 +261,8 @@ struct Wide {
 #pragma unroll
     for (int i = 0; i < K; ++i) a.a[i] = 0u;
   }
+  // a += b, both at the same exponent
+  __host__ __device__ static __forceinline__ void add_sum(sum& a, const u32* b) { add_words<K>(a.a, b); }
   // a += x y (neg = 0) or a -= x y (neg = ~0); E >= the product's exponent
   __host__ __device__ static __forceinline__ void mac(sum& a, int E, const num& x, const num& y, u32 neg) {
     u32 p[K];
