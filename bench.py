@@ -119,9 +119,10 @@ BATCHED = {
     "qd_batched_512": (4, 512, (16, 192), (0, 16)),
 }
 
-# FP64 pipe instructions of the kernels' primitives (static counts of csrc/ddqd.cuh):
-# complex conjugated multiply-accumulate, complex update y -= c x, |x|^2 accumulate,
-# complex / real division.
+# FP64 instructions of the primitives in error-free transforms (static counts of
+# csrc/ddqd.cuh): complex conjugated multiply-accumulate, complex update y -= c x, |x|^2
+# accumulate, complex / real division.  What a solve would cost on the FP64 pipe; complex
+# double runs on it.
 COST = {
     1: dict(mac=4, upd=4, norm=2, div=3),
     2: dict(mac=36, upd=42, norm=18, div=23),
@@ -130,6 +131,16 @@ COST = {
 # FP64 peak: 152 SMs x 4 sub-partitions x 0.5 FP64 lanes/clk (one DFMA warp-instruction
 # per 64 cycles per sub-partition, measured) at the 2070 MHz maximum SM clock.
 SMS, FP64_LANES_PER_CLK_SM = 152, 2.0
+
+# Double-double and quad-double run on integers (csrc/wide.cuh): 32 x 32 + 64-bit
+# multiply-adds of the same primitives, 10 and 28 a real product, 4 and 7 (and the digit's
+# own) a quotient digit of 28 bits.
+IMAD_COST = {
+    2: dict(mac=40, upd=40, norm=20, div=50),
+    4: dict(mac=112, upd=112, norm=56, div=144),
+}
+# Their peak: one warp-instruction per 4 clocks and sub-partition (measured).
+IMAD_LANES_PER_CLK_SM = 32.0
 
 
 L2_FLUSH_BYTES = 256 << 20  # twice the 129 MB L2
@@ -148,8 +159,35 @@ def flush_l2(dev):
 
 
 def fp64_ops(L: int, m: int, n: int) -> float:
-    """Algorithmic FP64 instructions (lane operations) of one solve."""
-    c = COST[L]
+    """Algorithmic FP64 instructions (lane operations) of one solve in error-free transforms."""
+    return _ops(COST[L], m, n)
+
+
+def alu_roofline(L: int, fp64: float, imad: float, seconds: float, sm_max_mhz: float, what: str) -> dict:
+    """The solve against the pipe it runs on: the FP64 pipe (complex double) or the integer
+    multiply-adds (double-double, quad-double), beside the FP64 instructions that limb arithmetic
+    would have taken in the same time over that pipe's peak (above 1 where it could not have
+    done the work)."""
+    fp64_peak = peak_fp64_ops_per_s(sm_max_mhz)
+    eq = {"instructions": fp64, "of_fp64_peak": fp64 / seconds / fp64_peak}
+    if L == 1:
+        return {"bound": "alu", "achieved": 2 * fp64 / seconds / 1e12, "peak": 2 * fp64_peak / 1e12, "unit": "TFLOP/s",
+                "frac": fp64 / seconds / fp64_peak, "fp64_equivalent": eq,
+                "note": "FP64 pipe: algorithmic FP64 instructions of %s (%.4g) / CUDA-event time; each one FMA slot "
+                        "(2 flops) like the peak (152 SMs x 2 DFMA/clk x %.0f MHz)" % (what, fp64, sm_max_mhz)}
+    peak = SMS * IMAD_LANES_PER_CLK_SM * sm_max_mhz * 1e6
+    return {"bound": "alu", "achieved": imad / seconds / 1e12, "peak": peak / 1e12, "unit": "T multiply-adds/s",
+            "frac": imad / seconds / peak, "fp64_equivalent": eq,
+            "note": "integer pipe: 32 x 32 + 64-bit multiply-adds of %s (%.4g) / CUDA-event time, peak 152 SMs x 32 "
+                    "lanes/clk x %.0f MHz" % (what, imad, sm_max_mhz)}
+
+
+def imad_ops(L: int, m: int, n: int) -> float:
+    """Algorithmic integer multiply-adds of one solve (0 for complex double)."""
+    return _ops(IMAD_COST[L], m, n) if L in IMAD_COST else 0.0
+
+
+def _ops(c: dict, m: int, n: int) -> float:
     nc = n + 1
     pairs = nc * (nc - 1) / 2  # (pivot k, column j > k) of the augmented matrix
     bulk = pairs * m * (c["mac"] + c["upd"])
@@ -169,7 +207,7 @@ def kernel_source_sha() -> str:
     import hashlib
 
     names = ["ddqd.cuh", "mgs_kernel.cuh", "mgs_cluster.cuh", "launch.cuh", "mgs_d.cu", "mgs_dd.cu", "mgs_qd.cu",
-             "api.cu"]
+             "wide.cuh", "wide_d.cuh", "mgs_column.cuh", "mgs_column.cu", "api.cu"]
     h = hashlib.sha256()
     for name in names:
         h.update(name.encode())
@@ -513,7 +551,6 @@ def run_gpu(args, L, m, n, extreme, rank, world):
     peaks = read_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     peak_ops = peak_fp64_ops_per_s(sm_max)
-    achieved_ops = ops / (kernel_ms / 1000.0)
     line = {
         "metric": METRIC, "value": value, "unit": "systems/s", "n_gpus": world, "steps": K, "warmup": W,
         "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -522,19 +559,15 @@ def run_gpu(args, L, m, n, extreme, rank, world):
         "e2e": {"value": world / (e2e_ms / 1000.0), "unit": "systems/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
         "gpu_launches": K,
-        "roofline": {"bound": "alu", "achieved": 2 * achieved_ops / 1e12, "peak": 2 * peak_ops / 1e12,
-                     "unit": "TFLOP/s", "frac": achieved_ops / peak_ops,
-                     "traffic": measured_traffic(args.workload),
-                     "note": "FP64 pipe: algorithmic FP64 instructions of the kernel's primitives per solve "
-                             "(%.4g) / CUDA-event time per solve; each instruction counted as one FMA slot "
-                             "(2 flops) like the peak (152 SMs x 2 DFMA/clk x %.0f MHz)" % (ops, sm_max)},
+        "roofline": dict(alu_roofline(L, ops, imad_ops(L, m, n), kernel_ms / 1000.0, sm_max, "a solve"),
+                         traffic=measured_traffic(args.workload)),
         "kernel_ms": kernel_ms,
         "cmac_rate": {"value": cmacs(L, m, n) / (kernel_ms / 1000.0) / 1e9, "unit": "G complex MAC/s",
                       "per_solve": cmacs(L, m, n),
                       "note": "m n (n + 1) complex multiply-accumulates of the projections and updates per "
                               "solve / CUDA-event time per solve; independent of the primitives' cost"},
         "hbm": {"bytes_per_solve": hbm_bytes(L, m, n), "achieved_gbs": hbm_bytes(L, m, n) / kernel_ms / 1e6,
-                "note": "algorithmic bytes / kernel time; the solve is FP64-bound, not HBM-bound"},
+                "note": "algorithmic bytes / kernel time; the solve is bound by its chain of steps, not by HBM"},
         "status_errors": len(bad),
     }
     if clk:
@@ -647,7 +680,6 @@ def run_gpu_batched(args, rank, world):
     peaks = read_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     peak_ops = peak_fp64_ops_per_s(sm_max)
-    achieved = ops / (kernel_ms / 1000.0)
     h2d = (base.A_pool.numel() + base.b_pool.numel()) * 8
     line = {
         "metric": METRIC, "value": value, "unit": "systems/s", "n_gpus": world, "steps": K, "warmup": W,
@@ -661,15 +693,14 @@ def run_gpu_batched(args, rank, world):
         "e2e": {"value": world * batch / (e2e_ms / 1000.0), "unit": "systems/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": base.x_pool.numel() * 8},
         "gpu_launches": K,
-        "roofline": {"bound": "alu", "achieved": 2 * achieved / 1e12, "peak": 2 * peak_ops / 1e12,
-                     "unit": "TFLOP/s", "frac": achieved / peak_ops, "traffic": measured_traffic(args.workload),
-                     "note": "FP64 pipe: algorithmic FP64 instructions of all systems (%.4g) per launch / "
-                             "CUDA-event time per launch" % ops},
+        "roofline": dict(alu_roofline(L, ops, sum(imad_ops(L, A.shape[1], A.shape[0]) for A, _ in host),
+                                      kernel_ms / 1000.0, sm_max, "all systems"),
+                         traffic=measured_traffic(args.workload)),
         "kernel_ms": kernel_ms,
         "cmac_rate": {"value": sum(cmacs(L, A.shape[1], A.shape[0]) for A, _ in host) / (kernel_ms / 1000.0) / 1e9,
                       "unit": "G complex MAC/s"},
         "sequential_plain": {"value": len(sel) / (seq_ms / 1000.0), "unit": "systems/s",
-                             "systems": len(sel), "frac": (seq_ops / (seq_ms / 1000.0)) / peak_ops,
+                             "systems": len(sel), "fp64_equivalent": (seq_ops / (seq_ms / 1000.0)) / peak_ops,
                              "note": "the same systems (every %d-th) solved one after another with the "
                                      "single-system solve on the same GPU" % max(1, batch // nseq)},
         "status_errors": bad,
@@ -789,8 +820,7 @@ def run_gpu_newton(args, rank, world):
     if rank != 0:
         return 0
     ops = S * fp64_ops(L, m, n)
-    peaks = read_peaks()
-    peak_ops = peak_fp64_ops_per_s(float(peaks.get("sm_max_mhz", 2070.0)))
+    sm_max = float(read_peaks().get("sm_max_mhz", 2070.0))
     line = {
         "metric": METRIC, "value": world * S / (ms / 1000.0), "unit": "Newton steps/s (one solve each)",
         "n_gpus": world, "steps": K, "warmup": W, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
@@ -801,9 +831,7 @@ def run_gpu_newton(args, rank, world):
         "e2e": {"value": world * S / (e2e_ms / 1000.0), "unit": "Newton steps/s",
                 "h2d_bytes_per_step": x0h.numel() * 8, "d2h_bytes_per_step": xh.numel() * 8 + sh.numel()},
         "gpu_launches": 3 * S * K,
-        "roofline": {"bound": "alu", "achieved": 2 * ops / (ms / 1000.0) / 1e12, "peak": 2 * peak_ops / 1e12,
-                     "unit": "TFLOP/s", "frac": ops / (ms / 1000.0) / peak_ops, "traffic": None,
-                     "note": "algorithmic FP64 instructions of the solves (%.4g) per run" % ops},
+        "roofline": dict(alu_roofline(L, ops, S * imad_ops(L, m, n), ms / 1000.0, sm_max, "the solves"), traffic=None),
         "eager_run_ms": eager_ms,
         "plain_solves_ms": solves_ms,
         "corrector_overhead": (ms - solves_ms) / solves_ms,
@@ -894,8 +922,7 @@ def run_gpu_diff(args, rank, world):
     if rank != 0:
         return 0
     ops = B * fp64_ops(L, m, n)
-    peaks = read_peaks()
-    peak_ops = peak_fp64_ops_per_s(float(peaks.get("sm_max_mhz", 2070.0)))
+    sm_max = float(read_peaks().get("sm_max_mhz", 2070.0))
     line = {
         "metric": METRIC, "value": world * B / (ms / 1000.0), "unit": "systems/s", "n_gpus": world, "steps": K,
         "warmup": W, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -906,9 +933,7 @@ def run_gpu_diff(args, rank, world):
                 "h2d_bytes_per_step": Ah.numel() * 8 + bh.numel() * 8,
                 "d2h_bytes_per_step": gAh.numel() * 8 + gbh.numel() * 8},
         "gpu_launches": 2 * K,
-        "roofline": {"bound": "alu", "achieved": 2 * ops / (ms / 1000.0) / 1e12, "peak": 2 * peak_ops / 1e12,
-                     "unit": "TFLOP/s", "frac": ops / (ms / 1000.0) / peak_ops, "traffic": None,
-                     "note": "algorithmic FP64 instructions of the forward solves only (%.4g) per step" % ops},
+        "roofline": dict(alu_roofline(L, ops, B * imad_ops(L, m, n), ms / 1000.0, sm_max, "the forward solves"), traffic=None),
         "forward_only": {"value": world * B / (fwd_ms / 1000.0), "unit": "systems/s", "ms": fwd_ms},
         "backward_overhead": (ms - fwd_ms) / fwd_ms,
     }

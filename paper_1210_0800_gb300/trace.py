@@ -13,13 +13,17 @@ wait for and copy of pivot k+1, partials of step k+1, grid barrier.  Of the clus
 schedule: the critical phases (a pivot applied to the next column a cluster publishes:
 on the owner of column k+1, and ahead of it on the owner of column k+2), then per bulk
 phase its Gram partials, cluster barrier and reduction, coefficient division, R/y stores
-and updates, and the wait for and copy of the next pivot.  Each phase is the per-step mean
-over the CTAs that ran it, summed over the steps.
+and updates, and the wait for and copy of the next pivot.  Of the kernel with whole columns
+per CTA: the wait for the pivot, and of the step's first pass (column k+1 alone on its owner)
+the dot products, the barrier, the sums over the warps and the division, the updates; then the
+other passes.  Each phase is the per-step mean over the CTAs that ran it, summed over the
+steps.
 """
 
 from __future__ import annotations
 
 import ctypes
+import os
 import sys
 
 import numpy as np
@@ -27,6 +31,7 @@ import numpy as np
 from . import _binding, build, inputs
 
 GRID_PHASES = ["reduce", "coef", "lookahead", "update", "wait+copy", "partials", "barrier"]
+COLUMN_PHASES = ["pivot wait", "dot products", "barrier", "sums+division", "updates", "other passes"]
 CLUSTER_PHASES = ["critical phases", "bulk partials", "barrier+reduce", "coef", "store+update", "pivot wait+copy"]
 
 
@@ -68,15 +73,22 @@ def summarize(plan, tr) -> str:
     """Per-phase sums of the per-step means over the CTAs active in the step."""
     nc = tr.shape[0] - 1
     sid = tr[0, :, 7]
-    lines = ["plan %s" % plan,
-             "CTAs %d on %d distinct SMs" % (len(sid), len(np.unique(sid)))]
+    lines = ["plan %s" % plan]
+    if sid.any():  # the kernel with whole columns does not record the SM
+        lines.append("CTAs %d on %d distinct SMs" % (len(sid), len(np.unique(sid))))
     grid = plan["kernel"] == "grid"
-    names = GRID_PHASES if grid else CLUSTER_PHASES
+    column = grid and plan["Br"] == 1 and not any(
+        v in os.environ for v in ("MGS_KERNEL", "MGS_ROWS", "MGS_CTA_THREADS", "MGS_CTAS_PER_SM"))
+    names = COLUMN_PHASES if column else GRID_PHASES if grid else CLUSTER_PHASES
     tot = np.zeros(len(names))
     for k in range(nc - 1 if grid else nc):
         row = tr[k]
         act = row[:, 0] > 0
-        if grid:
+        if column:
+            if act.any():
+                for i in range(len(names)):
+                    tot[i] += np.mean(row[act, i + 1] - row[act, i])
+        elif grid:
             if not act.any():
                 continue
             for i in range(len(names)):
@@ -112,6 +124,10 @@ def summarize(plan, tr) -> str:
     lines.append("sweep %.1f us, solve %.1f us" % ((ep[:, 0].max() - t0) / 1e3, (ep[:, 3].max() - t0) / 1e3))
     for nm, v in zip(names, tot):
         lines.append("  %-16s %9.1f us" % (nm, v / 1e3))
+    if column:
+        lines.append("  Q and R %.1f us, back substitution %.1f us" % (
+            np.mean(ep[:, 2] - ep[:, 1]) / 1e3, (ep[0, 3] - ep[0, 2]) / 1e3))
+        return "\n".join(lines)
     lines.append("  square roots %.1f us, Q and R scaling %.1f us, back substitution %.1f us" % (
         np.mean(ep[:, 1] - ep[:, 0]) / 1e3, np.mean(ep[:, 2] - ep[:, 1]) / 1e3, np.mean(ep[:, 3] - ep[:, 2]) / 1e3))
     return "\n".join(lines)
