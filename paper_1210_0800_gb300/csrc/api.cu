@@ -305,7 +305,7 @@ int run(int L, double* A, int lda, double* b, double* x, double* R, int ldr, dou
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* wb = static_cast<char*>(ws);
   cudaError_t e = cudaMemsetAsync(wb, 0, pl.zero_bytes, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dev_status, 0, sizeof(int32_t), st);
+  if (e == cudaSuccess && !pl.col) e = cudaMemsetAsync(dev_status, 0, sizeof(int32_t), st);  // the column kernel does
   if (e != cudaSuccess) {
     g_last_cuda = (int)e;
     return MGS_ECUDA;
