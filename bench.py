@@ -139,8 +139,9 @@ IMAD_COST = {
     2: dict(mac=40, upd=40, norm=20, div=50),
     4: dict(mac=112, upd=112, norm=56, div=144),
 }
-# Their peak: one warp-instruction per 4 clocks and sub-partition (measured).
-IMAD_LANES_PER_CLK_SM = 32.0
+# Their peak: one warp-instruction per 2 clocks and sub-partition (62.4 lanes per clock and SM
+# measured on independent chains of mad.wide.u32).
+IMAD_LANES_PER_CLK_SM = 64.0
 
 
 L2_FLUSH_BYTES = 256 << 20  # twice the 129 MB L2
@@ -178,7 +179,7 @@ def alu_roofline(L: int, fp64: float, imad: float, seconds: float, sm_max_mhz: f
     peak = SMS * IMAD_LANES_PER_CLK_SM * sm_max_mhz * 1e6
     return {"bound": "alu", "achieved": imad / seconds / 1e12, "peak": peak / 1e12, "unit": "T multiply-adds/s",
             "frac": imad / seconds / peak, "fp64_equivalent": eq,
-            "note": "integer pipe: 32 x 32 + 64-bit multiply-adds of %s (%.4g) / CUDA-event time, peak 152 SMs x 32 "
+            "note": "integer pipe: 32 x 32 + 64-bit multiply-adds of %s (%.4g) / CUDA-event time, peak 152 SMs x 64 "
                     "lanes/clk x %.0f MHz" % (what, imad, sm_max_mhz)}
 
 
