@@ -77,17 +77,18 @@ size_t mgs_workspace_bytes(int limbs, int m, int n, int with_rhs);
  * counterpart in the paper; for tests and tuning).  `out` has room for 5 ints.
  *   out[0] Br  row blocks (CTAs per column group), out[1] Bc  column groups,
  *   out[2] h   rows per row block, out[3] kernel:
- *     0  grid kernel: a plain cooperative grid.  Br = 1 (the default for limbs 2 and 4
- *        where a CTA's columns fit in shared memory): whole columns per CTA, integer
- *        arithmetic, no barrier between CTAs during the sweep.  Br > 1: row blocks, FP64
- *        arithmetic, one grid-wide barrier per elimination step;
+ *     0  grid kernel.  Br = 1 and h = m (the default where a CTA's columns fit in shared
+ *        memory): whole columns per CTA, integer arithmetic for limbs 2 and
+ *        4, no barrier between CTAs during the sweep; a cooperative grid, or clusters of 8
+ *        CTAs where a CTA owns at most two columns.  Else row blocks, FP64 arithmetic, a
+ *        plain cooperative grid, one grid-wide barrier per elimination step;
  *     1  cluster schedule on hardware thread-block clusters (the Br CTAs of a column
  *        group form one cluster and exchange Gram partials through distributed shared
  *        memory; Br <= 8);
  *     2  the same schedule on software groups (the Br CTAs meet at a counter in global
  *        memory and exchange partials through L2; every SM usable).
- *   Where whole columns do not fit, and for limbs 1, the default is 1 for limbs 1 and 2
- *   where the clusters fill at least 90 % of the SMs a plain grid would use, else 0.
+ *   Where whole columns do not fit, the default is 1 for limbs 1 and 2 where the clusters
+ *   fill at least 90 % of the SMs a plain grid would use, else 0.
  *   The environment variable MGS_KERNEL = grid | cluster | group, read at each call,
  *   forces a kernel with row blocks (cluster falls back to grid where clusters cannot be
  *   formed);

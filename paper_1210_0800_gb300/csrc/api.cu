@@ -178,7 +178,6 @@ bool compute_plan(int L, int m, int n, int aug, int want, int h0, int T0, int cp
 // stages fit in shared memory; the workspace stays at least what that plan asked for.
 void column_plan(Plan& pl) {
   const int L = pl.L, m = pl.m, nc = pl.nc;
-  if (m > 2048) return;
   const int sms = device_sms();
   const int bw = 1, first = 1;
   int stages = 4;

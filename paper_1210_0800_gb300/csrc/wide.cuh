@@ -1,8 +1,8 @@
 // Double-double and quad-double reals as wide binary floating-point numbers on the integer
 // pipe of sm_103a.
 //
-// Why: this GPU issues 2 FP64 lane-instructions per clock and SM, but 64 integer
-// multiply-adds (32 x 32 + 64 bits) and 64 integer adds, shifts and selects.  A
+// Why: this GPU issues 2 FP64 lane-instructions per clock and SM, but 62 integer
+// multiply-adds (32 x 32 + 64 bits) and 121 logical operations (measured).  A
 // quad-double product in error-free transforms is 70 FP64 instructions (2240 clocks of one
 // warp's sub-partition); the same product on 224-bit integers is 28 multiply-adds and about
 // 60 other instructions.  So inside the kernels a real is a sign, an exponent and an integer
@@ -156,7 +156,9 @@ struct Wide {
   static constexpr int K = W + 1;            // words of a product or a sum
   static constexpr int S = 2 * L;            // stored words
   static constexpr int BIAS = L == 2 ? 32768 : 1 << 20;
-  static constexpr int SUMBITS = 13;         // a sum may have up to 2^12 terms
+  // A sum may have 2^14 products: 2 m of them, with the m < 7300 whose pivot fits shared memory
+  // in the batched kernel.  The bits below are enough: a product is known to 124 (219) of 160 (256).
+  static constexpr int SUMBITS = 15;
 
   struct num {
     u32 m[W];

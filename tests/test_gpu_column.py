@@ -1,0 +1,100 @@
+"""The whole-column kernel and the batched kernel on integer arithmetic where their rules
+change: one row or column, remainders of 16 rows, column counts around a cluster, one and two
+columns a CTA, the tallest matrices, sums of as many near-equal terms as a column has, and back
+substitutions that no longer fit shared memory."""
+
+import numpy as np
+import pytest
+
+from helpers import compare_ls, gpu_ls_solve, gpu_qr, planted_system, rel, upper
+from paper_1210_0800_gb300 import inputs, mgs_plan_query
+
+pytestmark = pytest.mark.gpu
+
+U = {1: 2.0 ** -52, 2: 2.0 ** -104, 4: 2.0 ** -208}  # a few ulps: the bound of one operation
+
+
+def tolerance(A):
+    """An inner product of m terms is off by at most (m + 2) U of its terms; n of them follow
+    one another in a column, and the condition number multiplies what they leave in Q and x."""
+    n, m, _, L = A.shape
+    return 4 * (m + 2) * n * U[L] * np.linalg.cond(A[:, :, 0, 0] + 1j * A[:, :, 1, 0])
+
+
+def same_sign(m, n, L, seed):
+    """Parts in [0.98, 1): every product of a column has the same sign and nearly the largest
+    value that its exponent allows."""
+    A = inputs.matrix_uniform(m, n, L, seed)
+    A[..., 0] = 0.99 + 0.00999 * A[..., 0]
+    return A
+
+
+# (L, m, n): the columns with the right-hand side are n + 1
+SHAPES = [(1, 1, 1), (2, 1, 1), (4, 1, 1), (1, 17, 2), (2, 16, 7), (4, 33, 8), (2, 15, 15), (4, 49, 31), (2, 150, 143),
+          (1, 152, 151), (2, 152, 152), (1, 2048, 3), (2, 2048, 3), (4, 1000, 2), (4, 2048, 2)]
+
+
+@pytest.mark.parametrize("L,m,n", SHAPES)
+def test_column_kernel_vs_oracle_and_row_blocks(orc, monkeypatch, L, m, n):
+    monkeypatch.delenv("MGS_KERNEL", raising=False)
+    plan = mgs_plan_query(L, m, n, True)
+    # a quad-double column and two pivot stages no longer fit shared memory at 2048 rows
+    assert (plan["h"] == m) == (L < 4 or m <= 1000), plan
+    A, _, b = planted_system(m, n, L, 9100 + 3 * m + n + L, orc=orc)
+    tol = tolerance(A)
+    _, col, _ = compare_ls(orc, A, b, tol)
+    Qc, Rc, st = gpu_qr(A.copy())
+    assert st == 0
+    monkeypatch.setenv("MGS_KERNEL", "grid")
+    row = gpu_ls_solve(A.copy(), b.copy())
+    Qr, Rr, st = gpu_qr(A.copy())
+    assert st == 0 and row["status"] == 0
+    assert rel(orc, col["x"], row["x"]) <= tol
+    assert rel(orc, Qc, Qr) <= tol and rel(orc, upper(Rc), upper(Rr)) <= tol
+
+
+@pytest.mark.parametrize("L,m,n", [(2, 2048, 2), (4, 1000, 2)])
+def test_column_kernel_sums_of_one_sign(orc, L, m, n):
+    A = same_sign(m, n, L, 9300 + L)
+    b = orc.matvec(A, inputs.vector_uniform(n, L, 9301))
+    compare_ls(orc, A, b, tolerance(A))
+
+
+# the tallest systems of the batched kernel have about 7200 rows (DD) and 3500 (QD)
+@pytest.mark.parametrize("L,m,split", [(2, 2100, 1), (2, 6800, 1), (2, 6800, 2), (4, 3300, 1)])
+def test_batched_sums_of_one_sign(orc, L, m, split):
+    import torch
+
+    import paper_1210_0800_gb300 as mg
+
+    n = 3
+    A = same_sign(m, n, L, 9400 + m)
+    b = orc.matvec(A, inputs.vector_uniform(n, L, 9401))
+    bt = mg.make_batch([(A, b)], torch.device("cuda:0"))
+    st = mg.ls_solve_batched(bt, tune=(256, 1, split))
+    assert st.cpu().numpy().tolist() == [0]
+    o = orc.ls_solve(A.copy(), b.copy())
+    tol = tolerance(A)
+    assert rel(orc, bt.x_pool.cpu().numpy()[:n], o["x"]) <= tol
+    assert rel(orc, bt.A_pool.cpu().numpy()[: m * n].reshape(A.shape), o["Q"]) <= tol
+
+
+# sums and unknowns of the back substitution take 96 (DD) and 160 (QD) bytes an unknown, 64 KB at most
+@pytest.mark.parametrize("L,n", [(2, 682), (2, 683), (4, 409), (4, 410)])
+def test_batched_back_substitution_in_scratch(orc, L, n):
+    import torch
+
+    import paper_1210_0800_gb300 as mg
+
+    systems = []
+    for m, k in ((n, n), (40, 33)):
+        A, xt, _ = inputs.system(m, k, L, 9500 + m)
+        systems.append((A, orc.matvec(A, xt)))
+    bt = mg.make_batch(systems, torch.device("cuda:0"))
+    st = mg.ls_solve_batched(bt).cpu().numpy()
+    assert (st == 0).all()
+    for i, (A, b) in enumerate(systems):
+        g = gpu_ls_solve(A.copy(), b.copy())
+        k, xo = A.shape[0], int(bt.x_off[i])
+        assert g["status"] == 0
+        assert rel(orc, bt.x_pool[xo:xo + k].cpu().numpy(), g["x"]) <= tolerance(A)
