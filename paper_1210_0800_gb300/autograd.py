@@ -18,16 +18,23 @@ DEFAULT_SAVE_BUDGET = 1 << 30  # bytes of saved factors above which Q, R are rec
 
 
 def _uniform_batch(A, b):
-    """Batch view of uniform systems (copies into fresh pools: the solve overwrites them)."""
+    """Batch view of uniform systems (copies into fresh pools: the solve overwrites them).  Sizes
+    and offsets follow from the shape: one launch each and no read-back, which for small systems
+    cost more than their solve."""
     B, n, m, _, L = A.shape
     dev = A.device
-    ar = torch.arange(B, device=dev, dtype=torch.int64)
-    bt = _binding.Batch(A.reshape(B * n * m, 2, L).clone(), b.reshape(B * m, 2, L).clone(),
-                        torch.zeros((B * n, 2, L), dtype=torch.float64, device=dev),
-                        ar * (m * n), ar * m, ar * n,
-                        torch.full((B,), m, dtype=torch.int32, device=dev),
-                        torch.full((B,), n, dtype=torch.int32, device=dev), m, n)
-    return bt.with_R()
+    r = n * (n + 1) // 2
+
+    def offsets(step):
+        step = max(step, 1)
+        return torch.arange(0, B * step, step, device=dev, dtype=torch.int64)
+
+    return _binding.Batch(A.reshape(B * n * m, 2, L).clone(), b.reshape(B * m, 2, L).clone(),
+                          torch.zeros((B * n, 2, L), dtype=torch.float64, device=dev),
+                          offsets(m * n), offsets(m), offsets(n),
+                          torch.full((B,), m, dtype=torch.int32, device=dev),
+                          torch.full((B,), n, dtype=torch.int32, device=dev), m, n,
+                          R_pool=torch.zeros((B * r, 2, L), dtype=torch.float64, device=dev), r_off=offsets(r))
 
 
 def saved_bytes(B, m, n, L):
