@@ -45,9 +45,9 @@ bool make_bplan(int L, int batch, int max_m, int max_n, const mgs_tune* tune, BP
   } else if (wide) {
     // Split while a resident cluster would get fewer than two systems (its largest one is then
     // the launch's tail) and each CTA keeps 16 columns, or 8 while CTAs would stay idle.
-    // Double-double, ms at S = 1 / 2 / 4 with 304 resident CTAs: 512 systems of n <= 192 40 / 20.4 /
-    // 20.8, n <= 60 1.71 / 1.32 / 1.86, n <= 32 0.48 / 0.51 / 0.77; 1500 of n <= 64 4.1 / 5.2 / 7.2;
-    // 200 of n <= 120 7.5 / 5.1 / 3.3; 20 of n <= 40 0.51 / 0.38 / 0.29; 64 of n = 128 9.8 / 5.6 / 4.5
+    // Double-double, ms at S = 1 / 2 / 4 with 304 resident CTAs: 512 systems of n <= 192 37.4 / 20.1 /
+    // 19.4, n <= 60 1.62 / 1.22 / 1.78, n <= 32 0.46 / 0.49 / 0.77; 1500 of n <= 64 3.7 / 4.8 / 6.9;
+    // 200 of n <= 120 6.5 / 4.9 / 3.1; 20 of n <= 40 0.46 / 0.35 / 0.28; 64 of n = 128 8.9 / 5.0 / 4.2
     const long long slots = (long long)sms * bp.per_sm;
     bp.S = 1;
     while (bp.S < 4 && (long long)batch * bp.S < 2 * slots &&

@@ -3,22 +3,28 @@
 // (batched_kernel.cuh: Section 3, Figure 1 and Eq. 1; Section 6), organised for the integer
 // pipe.
 //
-// What bounds it: the integer multiply-adds of the products (a batch of hundreds of systems
-// fills the GPU), so no lane does what another lane has done:
+// What bounds it: instruction issue and the latency of the carry chains (four warps a scheduler,
+// 120 registers: half of the issue slots are busy; adds, shifts and selects 58 % of their pipe,
+// multiply-adds 17 %, DRAM 5 %), so no lane does what another lane has done:
 //   * A warp takes a trailing column through a whole step by itself -- dot product, division,
 //     update -- so a step has one barrier (the pivot's), and a warp reads its column twice
-//     in a row: the second time it is in L1.
+//     in a row: the second time it is in L1.  It takes two columns at a time: the pivot's words
+//     are read and unpacked once for both, their chains overlap, and one division, each column
+//     in its own eight lanes, serves both (ms, one column -> two: 512 DD 20.8 -> 20.0, 64 QD
+//     2.20 -> 1.94, 64 DD 160x128 with the adjoint 5.08 -> 4.81).
 //   * A lane owns one part of a row: lanes 0..15 the real parts of 16 rows, lanes 16..31 the
 //     imaginary parts.  The 32 lanes read 16 consecutive elements.
 //   * The pivot is staged in shared memory as planes of 16-byte words, its norm summed from
 //     the staging threads' own words.
 //   * The system is kept in its own memory as words (the bytes of the limbs): converted where
 //     the input is checked, converted back where Q is formed.
-// Measured, ms a batch, FP64 kernel before -> now: 512 DD systems of n <= 192 99.4 -> 20.5, 64 QD
-// systems of n <= 80 28.3 -> 1.9, 512 QD systems 728 -> 41.
+// Measured, ms a batch, FP64 kernel before -> now: 512 DD systems of n <= 192 99.4 -> 20.0, 64 QD
+// systems of n <= 80 28.3 -> 1.94, 512 QD systems 728 -> 41.
 // Split systems (S = 2 or 4 CTAs of a cluster): the columns are dealt out to the CTAs, which
 // meet once per step; only the pivot column is read by all of them.
 #pragma once
+
+#include <type_traits>
 
 #include "batched_kernel.cuh"
 #include "mgs_column.cuh"
@@ -49,6 +55,9 @@ __host__ __device__ inline long long batched_wide_scratch_doubles(int L, int max
                       (long long)batched_backsub_bytes(L, max_n) / 8;
   return (v + 31) / 32 * 32;
 }
+
+// Columns that a warp takes at a time (above).
+constexpr int kBatchedColumns = 2;
 
 template <int L, int T, int S>
 __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParams bp) {
@@ -195,67 +204,104 @@ __global__ void __launch_bounds__(T, 512 / T) mgs_batched_wide_kernel(BatchParam
       const bool ok = N::positive(g);
       if (!ok && tid == 0) sflag[1] = (sflag[1] == ST_OK) ? ST_ERANK : sflag[1];
       const num gn = N::unpack(g);
-      // column j > k: the own columns, one warp each
-      int j = k + 1 + ((rank - (k + 1)) % S + S) % S + warp * S;
-      for (; j < nc; j += NW * S) {
-        u32* cj = colw(j);
-        sum a;
-        int Ex = -4 * N::BIAS;
-        N::clear(a);
-        u32 v[SW], o[SW], vn[SW], on[SW];  // this piece's words, and the next one's, loaded ahead
-        {
+      // column j > k: the own columns, one warp for NC of them at a time
+      const int step = NW * S;
+      auto columns = [&](auto nc_const, int j) {
+        constexpr int NC = decltype(nc_const)::value;
+        u32* cj[NC];
+        sum a[NC];
+        int Ex[NC];
+        u32 v[NC][SW], o[SW], vn[NC][SW], on[NC][SW];  // this piece's words, and the next one's, loaded ahead
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          cj[c] = colw(j + c * step);
+          Ex[c] = -4 * N::BIAS;
+          N::clear(a[c]);
           const int l = min(lr, m - 1);
-          ld_part(cj + (size_t)(2 * l + part) * SW, vn);
-          ld_part(cj + (size_t)(2 * l + (part ^ 1)) * SW, on);
+          ld_part(cj[c] + (size_t)(2 * l + part) * SW, vn[c]);
+          ld_part(cj[c] + (size_t)(2 * l + (part ^ 1)) * SW, on[c]);
         }
         for (int l = lr; l < m; l += 16) {  // re: xr yr + xi yi, im: xr yi - xi yr
+          const num x1 = ld_num<L>(piv, m, l, 0), x2 = ld_num<L>(piv, m, l, 1);
+          const int ln = min(l + 16, m - 1);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+#pragma unroll
+            for (int i = 0; i < SW; ++i) {
+              v[c][i] = vn[c][i];
+              o[i] = on[c][i];
+            }
+            ld_part(cj[c] + (size_t)(2 * ln + part) * SW, vn[c]);
+            ld_part(cj[c] + (size_t)(2 * ln + (part ^ 1)) * SW, on[c]);
+            const num y1 = N::unpack(v[c]), y2 = N::unpack(o);
+            const int need = max(x1.e + y1.e, x2.e + y2.e) + N::SUMBITS;
+            if (need > Ex[c]) {
+              N::shift_sum(a[c], need - Ex[c]);
+              Ex[c] = need;
+            }
+            N::mac2(a[c], Ex[c], x1, y1, 0u, x2, y2, (u32)-part);
+          }
+        }
+        int top[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          top[c] = __reduce_max_sync(0xffffffffu, Ex[c]);
+          N::shift_sum(a[c], top[c] - Ex[c]);
+        }
+        // lanes with lr >= 8 of a pair go on with the last column's sum, so that one division serves all
+        const int mine = lr / (16 / NC);
+        if constexpr (NC == 2) {
+          u32 t[K];
+#pragma unroll
+          for (int q = 0; q < K; ++q) {
+            t[q] = __shfl_xor_sync(0xffffffffu, mine ? a[0].a[q] : a[1].a[q], 8);
+            a[0].a[q] = mine ? a[1].a[q] : a[0].a[q];
+          }
+          N::add_sum(a[0], t);
+          lane_sum<L, 3>(a[0]);
+        } else {
+          lane_sum<L, 4>(a[0]);
+        }
+        u32 f, q1[SW];
+        N::pack(N::quotient(N::normalize(a[0], mine ? top[NC - 1] : top[0], f), gn, f), f, q1);
+#pragma unroll
+        for (int i = 0; i < SW; ++i) q1[i] = ok ? q1[i] : 0u;
+        if (lr % (16 / NC) == 0) {
+          const int jm = j + mine * step;
+          st_part(((jm < n) ? Rp + packed(k, jm) * 2 * SW : Yv + (size_t)k * 2 * SW) + part * SW, q1);
+        }
+        num cr[NC], ci[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          u32 c1[SW], c2[SW];
 #pragma unroll
           for (int i = 0; i < SW; ++i) {
-            v[i] = vn[i];
-            o[i] = on[i];
+            c1[i] = __shfl_sync(0xffffffffu, q1[i], 8 * c);
+            c2[i] = __shfl_sync(0xffffffffu, q1[i], 16 + 8 * c);
           }
-          const int ln = min(l + 16, m - 1);
-          ld_part(cj + (size_t)(2 * ln + part) * SW, vn);
-          ld_part(cj + (size_t)(2 * ln + (part ^ 1)) * SW, on);
-          const num y1 = N::unpack(v), y2 = N::unpack(o);
-          const num x1 = ld_num<L>(piv, m, l, 0), x2 = ld_num<L>(piv, m, l, 1);
-          const int need = max(x1.e + y1.e, x2.e + y2.e) + N::SUMBITS;
-          if (need > Ex) {
-            N::shift_sum(a, need - Ex);
-            Ex = need;
-          }
-          N::mac2(a, Ex, x1, y1, 0u, x2, y2, (u32)-part);
-        }
-        const int top = __reduce_max_sync(0xffffffffu, Ex);
-        N::shift_sum(a, top - Ex);
-        lane_sum<L, 4>(a);
-        u32 f, c1[SW], c2[SW];
-        N::pack(N::quotient(N::normalize(a, top, f), gn, f), f, c1);
-#pragma unroll
-        for (int i = 0; i < SW; ++i) c1[i] = ok ? c1[i] : 0u;
-        if (lr == 0) st_part(((j < n) ? Rp + packed(k, j) * 2 * SW : Yv + (size_t)k * 2 * SW) + part * SW, c1);
-#pragma unroll
-        for (int i = 0; i < SW; ++i) {
-          const u32 t = c1[i];
-          c1[i] = __shfl_sync(0xffffffffu, t, 0);
-          c2[i] = __shfl_sync(0xffffffffu, t, 16);
-        }
-        const num cr = N::unpack(c1), ci = N::unpack(c2);
-        {
+          cr[c] = N::unpack(c1);
+          ci[c] = N::unpack(c2);
           const int l = min(lr, m - 1);
-          ld_part(cj + (size_t)(2 * l + part) * SW, vn);
+          ld_part(cj[c] + (size_t)(2 * l + part) * SW, vn[c]);
         }
         for (int l = lr; l < m; l += 16) {  // re: y - cr xr + ci xi, im: y - cr xi - ci xr
-#pragma unroll
-          for (int i = 0; i < SW; ++i) v[i] = vn[i];
+          const num x1 = ld_num<L>(piv, m, l, part), x2 = ld_num<L>(piv, m, l, part ^ 1);
           const int ln = min(l + 16, m - 1);
-          ld_part(cj + (size_t)(2 * ln + part) * SW, vn);
-          N::update(N::unpack(v), cr, ld_num<L>(piv, m, l, part), ~0u, ci, ld_num<L>(piv, m, l, part ^ 1), (u32)-part,
-                    v);
-          st_part(cj + (size_t)(2 * l + part) * SW, v);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+#pragma unroll
+            for (int i = 0; i < SW; ++i) v[c][i] = vn[c][i];
+            ld_part(cj[c] + (size_t)(2 * ln + part) * SW, vn[c]);
+            N::update(N::unpack(v[c]), cr[c], x1, ~0u, ci[c], x2, (u32)-part, v[c]);
+            st_part(cj[c] + (size_t)(2 * l + part) * SW, v[c]);
+          }
         }
         __syncwarp();
-      }
+      };
+      int j = k + 1 + ((rank - (k + 1)) % S + S) % S + warp * S;
+      for (; j + step * (kBatchedColumns - 1) < nc; j += step * kBatchedColumns)
+        columns(std::integral_constant<int, kBatchedColumns>{}, j);
+      if (j < nc) columns(std::integral_constant<int, 1>{}, j);
     }
     // r_kk
     if (lead) {
