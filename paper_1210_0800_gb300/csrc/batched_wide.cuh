@@ -4,7 +4,7 @@
 // pipe.
 //
 // What bounds it: instruction issue and the latency of the carry chains (four warps a scheduler,
-// 120 registers: half of the issue slots are busy; adds, shifts and selects 58 % of their pipe,
+// 126 registers: half of the issue slots are busy; adds, shifts and selects 58 % of their pipe,
 // multiply-adds 17 %, DRAM 5 %), so no lane does what another lane has done:
 //   * A warp takes a trailing column through a whole step by itself -- dot product, division,
 //     update -- so a step has one barrier (the pivot's), and a warp reads its column twice
