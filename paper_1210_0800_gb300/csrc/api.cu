@@ -53,9 +53,8 @@ struct Plan {
   int T;     // threads per CTA (128 or 256)
   size_t smem;
   size_t off_sync, off_gsync, off_flags, off_P, off_V, off_Y, off_R, off_G, off_T, total, zero_bytes;
-  // the column kernel (col != 0): panel width, warps on columns, pivot stages, column k+1 first,
-  // cluster size
-  int col, bw, warps, stages, first, CL;
+  // the column kernel (col != 0): warps on columns, pivot stages, cluster size
+  int col, warps, stages, CL;
   size_t off_C, off_Rd;
 };
 
@@ -179,7 +178,6 @@ bool compute_plan(int L, int m, int n, int aug, int want, int h0, int T0, int cp
 void column_plan(Plan& pl) {
   const int L = pl.L, m = pl.m, nc = pl.nc;
   const int sms = device_sms();
-  const int bw = 1, first = 1;
   int stages = 4;
   const int halves = (m + 15) / 16;  // 16-row pieces of a column
   // warps on columns: 15, or 12 where the pieces take no more rounds (two thirds of the warps in
@@ -192,7 +190,7 @@ void column_plan(Plan& pl) {
   // without: n = 32 DD 128 / 145, 256 DD 1413 / 1531, 320x256 QD 2253 / 2347; with more than two
   // columns a CTA the other columns' work hides the hand-off and the SMs that clusters leave
   // idle cost more: 512 QD 7710 / 7561.
-  const int w = (nc + sms - 1) / sms * bw;
+  const int w = (nc + sms - 1) / sms;
   int CL = w <= 2 ? 8 : 1;
   if (warps > halves * (w + 1)) warps = halves * (w + 1);  // a pass: w columns and the norm
   const int threads = 32 * (warps + 1);
@@ -221,10 +219,8 @@ void column_plan(Plan& pl) {
   pl.Bc = Bc;
   pl.h = m;
   pl.w = w;
-  pl.bw = bw;
   pl.warps = warps;
   pl.stages = stages;
-  pl.first = first;
   pl.CL = CL;
   pl.T = (nc + Bc - 1) / Bc >= 16 ? 256 : 128;
   pl.smem = smem;
@@ -323,11 +319,9 @@ int run(int L, double* A, int lda, double* b, double* x, double* R, int ldr, dou
     cp.nc = pl.nc;
     cp.aug = pl.aug;
     cp.Bc = pl.Bc;
-    cp.bw = pl.bw;
     cp.w = pl.w;
     cp.warps = pl.warps;
     cp.stages = pl.stages;
-    cp.first = pl.first;
     cp.CL = pl.CL;
     cp.C = reinterpret_cast<mgs::u32*>(wb + pl.off_C);
     cp.Rd = reinterpret_cast<mgs::u32*>(wb + pl.off_Rd);

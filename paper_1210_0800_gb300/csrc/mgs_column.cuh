@@ -6,8 +6,7 @@
 // k+1, which projects, divides, updates and passes pivot k+1 on; the other columns of a step
 // are work for a microsecond or two beside it.  So the layout takes off that chain what it
 // can:
-//   * A CTA owns panels of `bw` consecutive columns (cyclic over the CTAs), all rows, in
-//     shared memory.  A column's Gram entry needs no other CTA: no partial sums in global
+//   * A CTA owns columns c, c + Bc, ... (cyclic over the CTAs), all rows, in shared memory.  A column's Gram entry needs no other CTA: no partial sums in global
 //     memory and no barrier between CTAs in a step.
 //   * All warps of a CTA share its columns: a warp takes 16 rows of a column at a time, the
 //     real part in lanes 0..15 and the imaginary part in lanes 16..31 (the products of one
@@ -58,9 +57,8 @@ struct ColParams {
   double* x;
   double* z;
   int m, n, nc, aug;
-  int Bc, bw, w;          // CTAs, consecutive columns, slots per CTA
+  int Bc, w;              // CTAs, slots per CTA
   int warps, stages;      // warps that work on columns, pivot stages
-  int first;              // column k+1 goes before a step's other columns
   int CL;                 // CTAs of a cluster (1: none)
   u32* C;              // coefficients c_kj, k < j, packed: (j (j - 1) / 2 + k) * 2 S words
   u32* Rd;             // r_kk: nc * S words
@@ -366,7 +364,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   if (pr.skip && *pr.skip) return;  // uniform over the grid
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nthreads = blockDim.x;
-  const int c = blockIdx.x, Bc = pr.Bc, bw = pr.bw, m = pr.m, nc = pr.nc, w = pr.w;
+  const int c = blockIdx.x, Bc = pr.Bc, m = pr.m, nc = pr.nc, w = pr.w;
   const int NW = pr.warps, NS = pr.stages;
   extern __shared__ __align__(16) unsigned char csm[];
   const size_t colv = (size_t)L * m;  // uint4 per column
@@ -382,7 +380,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
   u64* empty = full + NS;                                        // all warps are done with it
   u64* pfull = empty + NS;                                       // a pushed pivot has arrived
   u64* pempty = pfull + 1;                                       // the CTA after has used the one pushed to it
-  auto col_of = [&](int s) { return ((s / bw) * Bc + c) * bw + s % bw; };
+  auto col_of = [&](int s) { return s * Bc + c; };
   auto gcol = [&](int j) { return (j < pr.n) ? pr.A + (size_t)j * pr.lda * E : pr.b; };
   int wc = 0;  // own columns
   while (wc < w && col_of(wc) < nc) ++wc;
@@ -427,7 +425,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     const int part = lane >> 4, lr = lane & 15;
     auto sync_warps = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(NW * 32) : "memory"); };
     // columns before jpub are followed by some column of another CTA
-    const int jpub = Bc == 1 ? 0 : jlast == nc - 1 ? jlast - jlast % bw : nc - 1;
+    const int jpub = Bc == 1 ? 0 : nc - 1;
     bool alive = true;
     u32 st = 0, turn = 0;  // the stage of the next pivot received, and its phase
     u32 pturn = 0;         // the phase of the next pushed pivot
@@ -435,7 +433,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
     int pushes = 0;        // pivots pushed to the CTA after
     const u32 rused = push_in ? peer_addr(pempty, crank - 1) : 0u;
     const u32 rpush = push_out ? peer_addr(push, crank + 1) : 0u, rbar = push_out ? peer_addr(pfull, crank + 1) : 0u;
-    int s0 = 0, next = wc > 0 ? c * bw : nc;  // the first own column not yet a pivot, and its slot
+    int s0 = 0, next = wc > 0 ? c : nc;  // the first own column not yet a pivot, and its slot
     const int kend = wc == 0 ? 0 : jlast == nc - 1 ? nc : jlast;  // the last column's owner ends with its norm
     // columns and warps of the last pass; the shares of a column in dots and in updates
     int pnb = -1, pnorm = -1, wpd = 1, cd = 0, sd = 0, wpu = 1, cu = 0, su = 0;
@@ -484,7 +482,7 @@ __global__ void __launch_bounds__(kColThreads, 1) mgs_column_kernel(ColParams pr
       bool norm = true;
       do {
         int nb = min(NW - 1, wc - sb);
-        if (crit && norm && pr.first) nb = 1;
+        if (crit && norm) nb = 1;
         if (nb != pnb || (int)norm != pnorm) {
           // a dot is two products a row and part, a norm one: the warps are shared 2 : 2 : .. : 1
           pnb = nb;
