@@ -31,10 +31,10 @@
 // keeps its rows as sums in shared memory, a link takes x_k off all of them and normalises
 // one, and the columns of coefficients arrive by bulk copies some links ahead.
 //
-// Measured, us a solve, row blocks on FP64 before -> now: DD 32x32 272 -> 118, 512x512 15423 -> 4600,
-// QD 65x64 2278 -> 330, 320x256 20331 -> 2210, 512x512 95627 -> 7660, complex double 128x128
-// 615 -> 471.  Of QD 320x256, the sweep is 1960 (pivot wait 330, dot products 590, sums and
-// division 350, updates 620), the back substitution 250.
+// Measured, us a solve, row blocks on FP64 before -> now: DD 32x32 271 -> 116, 512x512 15453 ->
+// 4490, QD 65x64 2285 -> 326, 320x256 20364 -> 2142, 512x512 95763 -> 7439, complex double 128x128
+// 612 -> 442.  Of QD 320x256, the sweep is 1910 (pivot wait 330, dot products 590, sums and
+// division 330, updates 590), the back substitution 250.
 //
 // Every wait is bounded: after the time limit it records a timeout status and raises the
 // abort flag, and all later waits fall through.
